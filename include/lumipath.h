@@ -101,8 +101,9 @@ typedef struct lf_launch {
     uint32_t tile_h;           /* pixels per CTA tile in y; power of two, multiple of 32/warp_w */
     uint32_t warp_w;           /* 1, 2, 4, 8, 16 or 32 */
     uint32_t order;            /* 0: tiles in raster order per view; 1: strips of 4 tile rows, column by column */
-    uint32_t persistent;       /* 0: one CTA per tile; 1: CTAs pull tiles from a queue */
-    uint32_t ctas_per_sm;      /* persistent grid = SMs * ctas_per_sm (0: occupancy) */
+    uint32_t persistent;       /* 0 or 1: no effect (a launch has one CTA per tile, and the
+                                  hardware's block scheduler is its queue) */
+    uint32_t ctas_per_sm;      /* no effect */
 } lf_launch;
 
 typedef struct lf_table lf_table;
@@ -330,9 +331,9 @@ lf_status lf_post_filter(double radius, const double center[3], uint32_t channel
  * and idx_dev as for lf_render; launch may be NULL for the default shape). It
  * writes the same image and indices as lf_create_table + lf_render.
  * The SF point caches, the status/queue words and the queue of rays left to
- * the exact pass live in one fixed device array inside the library (32 B per
+ * the exact pass live in one fixed device array inside the library (48 B per
  * point for up to LF_NOALLOC_MAX_POINTS points plus 8 B per queued ray for up
- * to LF_NOALLOC_MAX_DEFERRED rays, about 8.6 MiB), which every GPU that loads
+ * to LF_NOALLOC_MAX_DEFERRED rays, about 12.9 MiB), which every GPU that loads
  * the library keeps until the process exits. Each call rebuilds that content
  * on `stream` and leaves the last call's contents behind; calls that overlap
  * on the GPU (other streams or threads) race on it. Every call looks up the

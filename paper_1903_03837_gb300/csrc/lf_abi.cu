@@ -184,7 +184,39 @@ ViewK view_params(const lf_view &w, const lf_launch &L, double R, const double O
     k.tiles_x = (w.width + L.tile_w - 1) / L.tile_w;
     k.tiles_y = (w.height + L.tile_h - 1) / L.tile_h;
     fill_view_miss_consts(k, R, O);
+    fill_certain_miss(k);
+    fill_screen_bound(k);
+    // division by tiles_x of a dividend below 2^31: ceil(2^(31 + l) / d), l = ceil(log2 d)
+    // (Granlund and Montgomery, "Division by invariant integers using multiplication")
+    uint32_t l = 0;
+    while ((1u << l) < k.tiles_x) ++l;
+    k.div_s = 31 + l;
+    k.div_m = (uint32_t)(((1ull << (31 + l)) + k.tiles_x - 1) / k.tiles_x);
     return k;
+}
+
+PointSetK point_set_of(const float4 *hi, const float4 *lo, const float4 *xy, uint32_t n)
+{
+    const double sigma2 = 12.566370614359172953850573533118 / (double)n, step = 2.0 / (double)n;
+    PointSetK P;
+    P.hi = hi;
+    P.lo = lo;
+    P.xy = xy;
+    P.n = n;
+    P.nf = (float)n;
+    P.inv_sigma = (float)(1.0 / std::sqrt(sigma2));
+    P.sigma2 = (float)sigma2;
+    P.zone0 = (float)(std::log(std::sqrt(5.0) * 3.14159265358979323846 * n) / (2.0 * std::log(1.6180339887498948482)));
+    P.zstep_h = (float)step;
+    P.zstep_l = (float)(step - (double)P.zstep_h);
+    P.zhalf = (float)(0.5 * step);
+    return P;
+}
+
+uint64_t table_bytes_of(int kind, uint32_t rows, uint32_t N)
+{
+    const uint64_t texel = kind == kF32C4 ? 16 : kind == kF32C3 ? 12 : kind == kF16C4 ? 8 : 4;
+    return (uint64_t)rows * N * texel;
 }
 
 // Checks of a table description shared by lf_create_table and
@@ -236,21 +268,10 @@ lf_status run_chunk(const lf_table *t, const lfk::RenderParamsBase &base, const 
     p.total_tiles = (uint32_t)tiles;
     p.total_pixels = 0;
     for (uint32_t v = 0; v < nv; ++v) p.total_pixels += (uint64_t)views[v].width * views[v].height;
-    unsigned block = L.tile_w * L.tile_h;
-    unsigned grid = (unsigned)tiles;
-    if (L.persistent) {
-        int per_sm = L.ctas_per_sm ? (int)L.ctas_per_sm
-                                   : lfk::render_occupancy(t->texel_kind, bwd, MAXV != lfk::kSmallViews,
-                                                           p.nine != 0, block);
-        uint64_t g = (uint64_t)t->sm_count * (uint64_t)per_sm;
-        grid = (unsigned)(g < tiles ? g : tiles);
-    }
+    const unsigned block = L.tile_w * L.tile_h, grid = (unsigned)tiles;
     if (grid == 0) return LF_OK;
-    cudaError_t e;
-    if constexpr (MAXV == lfk::kSmallViews)
-        e = lfk::launch_render_small(t->texel_kind, bwd, p, grid, block, st);
-    else
-        e = lfk::launch_render_large(t->texel_kind, bwd, p, grid, block, st);
+    const cudaError_t e = bwd ? lfk::launch_backward(p, grid, block, st)
+                              : lfk::launch_render(t->texel_kind, p, grid, block, st);
     if (e != cudaSuccess) return cuda_fail(e, bwd ? "backward launch" : "render launch");
     return LF_OK;
 }
@@ -286,8 +307,6 @@ lf_status run(const lf_table *t, const lf_view *views, uint32_t n_views, float *
     b.grad_out = grad_out;
     b.grad = grad;
     b.status = t->scratch;
-    b.queue = t->scratch + 1;
-    b.done = t->scratch + 2;
     b.defer_done = t->scratch + 3;
     b.defer_count = reinterpret_cast<unsigned long long *>(t->scratch + 4);
     b.defer_items = reinterpret_cast<unsigned long long *>(reinterpret_cast<char *>(t->scratch) + lfk::kWordsBytes);
@@ -296,11 +315,11 @@ lf_status run(const lf_table *t, const lf_view *views, uint32_t n_views, float *
     b.tile_h = t->launch.tile_h;
     b.warp_w = t->launch.warp_w;
     b.order = t->launch.order;
-    b.persistent = t->launch.persistent;
     b.tw_log = (uint32_t)__builtin_ctz(t->launch.tile_w);
     b.th_log = (uint32_t)__builtin_ctz(t->launch.tile_h);
     b.ww_log = (uint32_t)__builtin_ctz(t->launch.warp_w);
     b.rows_valid = t->rows;
+    b.table_bytes = lfk::table_bytes_of(t->texel_kind, t->rows, t->desc.n_directions);
     b.nearest_only = t->desc.k_nearest == 1 ? 1u : 0u;
     b.nine = t->desc.k_nearest == 9 ? 1u : 0u;
     b.rows_stored = (t->desc.flags & LF_TABLE_UPPER_HEMISPHERE) ? t->rows : 0u;
@@ -322,6 +341,50 @@ size_t code_bytes(int dtype) { return dtype == LF_DTYPE_F32 ? 4 : (dtype == LF_D
 namespace lfk {
 void set_last_error(const char *msg) { g_err = msg ? msg : ""; }
 
+// The form (1 + m) (f0 . v)(f0 . w) - (1 - m) c0 v.w over the view's image-plane
+// basis: v(x, y) = F + x A + y B is the ray of image-plane coordinates x, y in
+// [-1, 1] (y up), V = (F, A, B). A ray of S[.][.] < 0 misses S by the relative
+// margin m.
+static void miss_form(const ViewK &k, double m, double S[3][3])
+{
+    double V[3][3], f[3];
+    for (int i = 0; i < 3; ++i) {
+        V[0][i] = k.fwd[i];
+        V[1][i] = (double)k.tan_x * k.right[i];
+        V[2][i] = (double)k.tan_y * k.up[i];
+    }
+    for (int a = 0; a < 3; ++a) f[a] = (double)k.f0[0] * V[a][0] + (double)k.f0[1] * V[a][1] + (double)k.f0[2] * V[a][2];
+    for (int a = 0; a < 3; ++a)
+        for (int b = 0; b < 3; ++b)
+            S[a][b] = (1.0 + m) * f[a] * f[b] -
+                      (1.0 - m) * (double)k.c0 * (V[a][0] * V[b][0] + V[a][1] * V[b][1] + V[a][2] * V[b][2]);
+}
+
+// Coefficients of certain_miss: the form in pixel coordinates, raised by its
+// FP32 rounding (at most 12 * 2^-24 of the terms' magnitudes over the view; 2^-20
+// taken). Without an eye clearly outside S, or where FP32 does not hold the
+// coefficients, no ray misses certainly.
+void fill_certain_miss(ViewK &k)
+{
+    k.q[0] = 1.0f;
+    for (int i = 1; i < 6; ++i) k.q[i] = 0.0f;
+    if (!k.outside) return;
+    double S[3][3];
+    miss_form(k, 1e-4, S);
+    // x = sx px + tx, y = sy py + ty
+    const double sx = 2.0 / k.width, tx = 1.0 / k.width - 1.0, sy = -2.0 / k.height, ty = 1.0 - 1.0 / k.height;
+    double q[6] = {S[0][0] + 2.0 * S[0][1] * tx + 2.0 * S[0][2] * ty + S[1][1] * tx * tx + 2.0 * S[1][2] * tx * ty + S[2][2] * ty * ty,
+                   2.0 * sx * (S[0][1] + S[1][1] * tx + S[1][2] * ty), 2.0 * sy * (S[0][2] + S[1][2] * tx + S[2][2] * ty),
+                   S[1][1] * sx * sx, 2.0 * S[1][2] * sx * sy, S[2][2] * sy * sy};
+    const double W = k.width, H = k.height;
+    const double mag = std::fabs(q[0]) + W * (std::fabs(q[1]) + W * std::fabs(q[3])) +
+                       H * (std::fabs(q[2]) + H * std::fabs(q[5]) + W * std::fabs(q[4]));
+    q[0] += std::ldexp(mag, -20);
+    for (int i = 0; i < 6; ++i)
+        if (!(std::fabs(q[i]) < 1e37) || !(mag > 1e-30)) return;
+    for (int i = 0; i < 6; ++i) k.q[i] = (float)q[i];
+}
+
 void fill_view_miss_consts(ViewK &k, double R, const double O[3])
 {
     double f[3] = {(double)k.eye[0] - O[0], (double)k.eye[1] - O[1], (double)k.eye[2] - O[2]};
@@ -330,6 +393,41 @@ void fill_view_miss_consts(ViewK &k, double R, const double O[3])
     k.ff0 = (float)ff;
     k.c0 = (float)(ff - R * R);
     k.outside = (ff - R * R) > 1e-3 * ff ? 1u : 0u;
+}
+
+// Columns [sx0, sx1) and rows [sy0, sy1) outside which every pixel certainly
+// misses S: the form's zero set, when it is an ellipse, is bounded by where its
+// discriminant in the other coordinate vanishes. Twice the margin of
+// certain_miss here and three pixels more cover every rounding; anything but an
+// ellipse bounds nothing.
+void fill_screen_bound(ViewK &k)
+{
+    k.sx0 = k.sy0 = 0;
+    k.sx1 = k.width;
+    k.sy1 = k.height;
+    if (!k.outside) return;
+    double S[3][3];
+    miss_form(k, 2e-4, S);
+    // extent of coordinate u (1: x, 2: y): the roots of the discriminant in w = 3 - u
+    double lo[3], hi[3];
+    for (int u = 1; u <= 2; ++u) {
+        const int w = 3 - u;
+        const double A = S[u][w] * S[u][w] - S[w][w] * S[u][u], B = S[0][w] * S[u][w] - S[w][w] * S[0][u],
+                     C = S[0][w] * S[0][w] - S[w][w] * S[0][0], disc = B * B - A * C;
+        if (!(S[w][w] < 0.0 && A < 0.0 && disc > 0.0)) return;
+        const double r = std::sqrt(disc);
+        lo[u] = (-B + r) / A;          // A < 0: the smaller root
+        hi[u] = (-B - r) / A;
+        if (!(lo[u] <= hi[u]) || !std::isfinite(lo[u]) || !std::isfinite(hi[u])) return;
+    }
+    auto pixel = [](double t, uint32_t n, int grow) {      // clamped pixel coordinate of t in [-1, 1]
+        const double px = std::floor((t + 1.0) * 0.5 * n) + grow;
+        return (uint32_t)(px < 0.0 ? 0.0 : px > (double)n ? (double)n : px);
+    };
+    k.sx0 = pixel(lo[1], k.width, -3);
+    k.sx1 = pixel(hi[1], k.width, 4);
+    k.sy0 = pixel(-hi[2], k.height, -3);                   // row 0 is y = +1
+    k.sy1 = pixel(-lo[2], k.height, 4);
 }
 
 void fill_sphere_consts(SphereK &S, double R, const double O[3])
@@ -418,14 +516,15 @@ lf_status lf_create_table(const lf_table_desc *d, const void *radiance_dev, cons
     cudaError_t e;
     auto bail = [&](lf_status s) { lf_destroy(t); return s; };
 
-    e = cudaMalloc(&t->points, sizeof(float4) * 2ull * ((uint64_t)M + N));
+    e = cudaMalloc(&t->points, sizeof(float4) * (3ull * ((uint64_t)M + N) + 4ull * lfk::kPointPad));
     if (e != cudaSuccess) return bail(cuda_fail(e, "point cache allocation"));
     e = cudaMalloc(&t->scratch, lfk::kWordsBytes + sizeof(unsigned long long) * (size_t)lfk::kDeferCap);
     if (e != cudaSuccess) return bail(cuda_fail(e, "scratch allocation"));
     e = cudaMemsetAsync(t->scratch, 0, lfk::kWordsBytes, st);
     if (e != cudaSuccess) return bail(cuda_fail(e, "scratch clear"));
-    e = lfk::launch_build_points(M, t->points, t->points + M, st);
-    if (e == cudaSuccess) e = lfk::launch_build_points(N, t->points + 2 * (uint64_t)M, t->points + 2 * (uint64_t)M + N, st);
+    float4 *po = t->points, *pd = t->points + 3 * (uint64_t)M + 2 * lfk::kPointPad;
+    e = lfk::launch_build_points(M, po, po + M, po + 2 * (uint64_t)M, st);
+    if (e == cudaSuccess) e = lfk::launch_build_points(N, pd, pd + N, pd + 2 * (uint64_t)N, st);
     if (e != cudaSuccess) return bail(cuda_fail(e, "point cache build"));
 
     if (!quant) t->texel_kind = C == 4 ? lfk::kF32C4 : lfk::kF32C3;
@@ -456,10 +555,8 @@ lf_status lf_create_table(const lf_table_desc *d, const void *radiance_dev, cons
 
     lfk::SphereK &S = t->sphere;
     lfk::fill_sphere_consts(S, d->radius, d->center);
-    const double four_pi = 12.566370614359172953850573533118;
-    t->po = {t->points, t->points + M, M, (float)M, (float)(1.0 / std::sqrt(four_pi / (double)M))};
-    t->pd = {t->points + 2 * (uint64_t)M, t->points + 2 * (uint64_t)M + N, N, (float)N,
-             (float)(1.0 / std::sqrt(four_pi / (double)N))};
+    t->po = lfk::point_set_of(po, po + M, po + 2 * (uint64_t)M, M);
+    t->pd = lfk::point_set_of(pd, pd + N, pd + 2 * (uint64_t)N, N);
     *out = t;
     return LF_OK;
 }
@@ -594,11 +691,10 @@ lf_status lf_fill_lobe_table(uint32_t M, uint32_t N, uint32_t C, uint32_t L, con
     float4 *pts = nullptr;
     cudaError_t e = cudaMallocAsync((void **)&pts, sizeof(float4) * 2ull * ((uint64_t)M + N), st);
     if (e != cudaSuccess) return cuda_fail(e, "point allocation");
-    e = lfk::launch_build_points(M, pts, pts + M, st);
-    if (e == cudaSuccess) e = lfk::launch_build_points(N, pts + 2 * (uint64_t)M, pts + 2 * (uint64_t)M + N, st);
-    if (e == cudaSuccess)
-        e = lfk::launch_fill_lobe(P, pts, pts + M, pts + 2 * (uint64_t)M, pts + 2 * (uint64_t)M + N, M, N,
-                                  out_dev, st);
+    float4 *pd = pts + 2 * (uint64_t)M;
+    e = lfk::launch_build_points(M, pts, pts + M, nullptr, st);
+    if (e == cudaSuccess) e = lfk::launch_build_points(N, pd, pd + N, nullptr, st);
+    if (e == cudaSuccess) e = lfk::launch_fill_lobe(P, pts, pts + M, pd, pd + N, M, N, out_dev, st);
     cudaError_t e2 = cudaFreeAsync(pts, st);
     if (e != cudaSuccess) return cuda_fail(e, "lobe fill");
     if (e2 != cudaSuccess) return cuda_fail(e2, "point free");
@@ -630,12 +726,13 @@ lf_status lf_precompute_table(const lf_precompute_desc *d, const lf_blob *blobs,
     float4 *pts = nullptr;
     cudaError_t e = cudaMallocAsync((void **)&pts, sizeof(float4) * 2ull * ((uint64_t)M + N), st);
     if (e != cudaSuccess) return cuda_fail(e, "point allocation");
+    float4 *pd = pts + 2 * (uint64_t)M;
     P.po_hi = pts;
     P.po_lo = pts + M;
-    P.pd_hi = pts + 2 * (uint64_t)M;
-    P.pd_lo = pts + 2 * (uint64_t)M + N;
-    e = lfk::launch_build_points(M, pts, pts + M, st);
-    if (e == cudaSuccess) e = lfk::launch_build_points(N, pts + 2 * (uint64_t)M, pts + 2 * (uint64_t)M + N, st);
+    P.pd_hi = pd;
+    P.pd_lo = pd + N;
+    e = lfk::launch_build_points(M, pts, pts + M, nullptr, st);
+    if (e == cudaSuccess) e = lfk::launch_build_points(N, pd, pd + N, nullptr, st);
     if (e == cudaSuccess) e = lfk::launch_precompute(P, st);
     cudaError_t e2 = cudaFreeAsync(pts, st);
     if (e != cudaSuccess) return cuda_fail(e, "precompute");

@@ -21,30 +21,59 @@ namespace lfk {
 // coordinates has basis (eps_k, F_k), (eps_{k+1}, F_{k+1}).
 // ---------------------------------------------------------------------------
 constexpr int kFibN = 40;
-struct FibTables {
-    int32_t F[kFibN];
-    float eps[kFibN];
+// Per zone k: the coefficients of the lattice coordinates u = au t + bu i_c,
+// v = av t + bv i_c (t the azimuth in turns, i_c the continuous index), that is
+// sg (-F_{k+1} t + eps_{k+1} i_c) and sg (F_k t - eps_k i_c) with sg = -1 for odd
+// k, and F_k, F_{k+1}.
+struct __align__(16) LatticeZone {
+    float au, bu, av, bv;
+    int32_t F0, F1, pad0, pad1;
 };
-constexpr FibTables make_fib() {
-    FibTables t{};
-    long long a = 0, b = 1;
-    double g = 0.61803398874989484820, gk = 1.0;
+struct LatticeZones {
+    LatticeZone z[kFibN - 2];
+};
+constexpr LatticeZones make_zones() {
+    long long F[kFibN] = {0, 1};
+    double eps[kFibN] = {}, gk = 1.0;
     for (int k = 0; k < kFibN; ++k) {
-        t.F[k] = (int32_t)a;
-        long long c = a + b;
-        a = b;
-        b = c;
-        t.eps[k] = (float)((k % 2 == 1) ? gk : -gk);   // (-1)^(k+1) g^k
-        gk *= g;
+        if (k >= 2) F[k] = F[k - 1] + F[k - 2];
+        eps[k] = k % 2 == 1 ? gk : -gk;                // (-1)^(k+1) Phi^-k
+        gk *= 0.61803398874989484820;
+    }
+    LatticeZones t{};
+    for (int k = 0; k < kFibN - 2; ++k) {
+        const double sg = k % 2 == 1 ? -1.0 : 1.0;
+        t.z[k].au = (float)(-sg * (double)F[k + 1]);
+        t.z[k].bu = (float)(sg * eps[k + 1]);
+        t.z[k].av = (float)(sg * (double)F[k]);
+        t.z[k].bv = (float)(-sg * eps[k]);
+        t.z[k].F0 = (int32_t)F[k];
+        t.z[k].F1 = (int32_t)F[k + 1];
     }
     return t;
 }
-__constant__ constexpr FibTables kFib = make_fib();
+__constant__ constexpr LatticeZones kZones = make_zones();
 
-// log2(Phi^2), used by the zone number k = floor(log_{Phi^2}(sqrt5*pi*n*(1-z^2))).
+// The zone number is k = floor(log_{Phi^2}(sqrt5*pi*n*(1-z^2))) = floor(
+// log2(1-z^2) / log2(Phi^2) + zone0), zone0 the set's part (PointSetK).
 constexpr float kInvLog2Phi2 = 0.72021234840458929f;    // 1 / log2(Phi^2)
-constexpr float kSqrt5Pi = 7.0248147310407731f;          // sqrt(5)*pi
 constexpr float kInv2Pi = 0.15915494309189535f;
+
+// Hardware approximations (relative error below 2^-22; arguments here are never
+// denormal): the functions of the same name spend two to four instructions more
+// on denormals.
+__device__ __forceinline__ float lg2_approx(float x)
+{
+    float r;
+    asm("lg2.approx.ftz.f32 %0, %1;" : "=f"(r) : "f"(x));
+    return r;
+}
+__device__ __forceinline__ float sqrt_approx(float x)
+{
+    float r;
+    asm("sqrt.approx.ftz.f32 %0, %1;" : "=f"(r) : "f"(x));
+    return r;
+}
 
 // Azimuth of (x, y) in turns, for choosing the lattice cell only. atan on
 // [0, 1] is a degree-15 odd polynomial, minimax over [0, 1] (Lawson's
@@ -132,30 +161,22 @@ __device__ __forceinline__ bool intersect_sphere(const SphereK &S, const float e
     return true;
 }
 
-// True only for rays that certainly miss S: an approximate ray (FMA, no IEEE
-// division) whose line passes outside S, or points away from it, by a
-// relative margin of 1e-4 -- far beyond the ~1e-6 difference between this
-// approximation and the exact FP32 ray, so the exact step would also report a
-// miss. Anything else takes the exact path.
-__device__ __forceinline__ bool certain_miss(const ViewK &v, uint32_t x, uint32_t y)
+// True only for rays that certainly miss S: the discriminant (f0.v)^2 - c0 v.v of
+// the unnormalised ray v is a quadratic in the pixel's coordinates, with
+// coefficients that carry a relative margin of 1e-4 -- far beyond the ~1e-6
+// difference to the exact FP32 ray -- and the quadratic's own FP32 rounding
+// (fill_certain_miss), so the exact step would also report a miss. Anything
+// else takes the exact path. Eight instructions, where the ray itself took 35.
+__device__ __forceinline__ bool certain_miss(const ViewK &v, uint32_t px, uint32_t py)
 {
-    if (!v.outside) return false;
-    float nx = __fmaf_rn(__uint2float_rn(x) + 0.5f, v.inv2w, -1.0f) * v.tan_x;
-    float ny = __fmaf_rn(-(__uint2float_rn(y) + 0.5f), v.inv2h, 1.0f) * v.tan_y;
-    float vx = __fmaf_rn(ny, v.up[0], __fmaf_rn(nx, v.right[0], v.fwd[0]));
-    float vy = __fmaf_rn(ny, v.up[1], __fmaf_rn(nx, v.right[1], v.fwd[1]));
-    float vz = __fmaf_rn(ny, v.up[2], __fmaf_rn(nx, v.right[2], v.fwd[2]));
-    float b = __fmaf_rn(v.f0[0], vx, __fmaf_rn(v.f0[1], vy, v.f0[2] * vz));
-    float vv = __fmaf_rn(vx, vx, __fmaf_rn(vy, vy, vz * vz));
-    float b2 = b * b, vc = vv * v.c0;
-    bool no_disc = (b2 - vc) < -1e-4f * (b2 + vc);
-    // b > 1e-4 |v| |f0|, compared in squares (no square root)
-    bool away = b > 0.0f && b2 > 1e-8f * (vv * v.ff0);
-    return no_disc || away;
+    const float x = __uint2float_rn(px), y = __uint2float_rn(py);
+    const float a = __fmaf_rn(v.q[3], x, __fmaf_rn(v.q[4], y, v.q[1]));
+    const float b = __fmaf_rn(v.q[5], y, v.q[2]);
+    return __fmaf_rn(x, a, __fmaf_rn(y, b, v.q[0])) < 0.0f;
 }
 
-// The hit mask of a pixel's ray by the approximate ray of certain_miss, where
-// it is certain: 0 if the ray certainly misses S, 1 if it certainly hits S in
+// The hit mask of a pixel's ray by an approximate ray (FMA, no IEEE division),
+// where it is certain: 0 if the ray certainly misses S, 1 if it certainly hits S in
 // front of the eye (discriminant above 0 and direction towards the centre,
 // both by the relative margin 1e-4, so the exact step would report the same),
 // -1 if only the exact ray/sphere step can tell.
@@ -423,28 +444,40 @@ __device__ __forceinline__ int32_t source_index(const Source &s, uint32_t slot)
 // with the lattice coordinates and the zone perturbed by more than their FP32
 // error). Outside the pole scan the zone is k >= 6 (F_k >= 8), so the 12
 // corners have distinct indices.
-__device__ __forceinline__ Source lattice_window(const PointSetK &P, float3 qh)
+struct Corner {
+    int32_t b, G0, G1;       // the rounded corner's index and the quadrant's basis
+    int32_t reach;           // F_k + F_{k+1}
+};
+__device__ __forceinline__ Corner lattice_corner(const PointSetK &P, float3 qh)
 {
     float z = qh.z;
     float omz2 = __fmul_rn(__fsub_rn(1.0f, z), __fadd_rn(1.0f, z));
     float t = azimuth_turns(qh.y, qh.x);                            // turns
     float ic = (P.nf * (1.0f - z) - 1.0f) * 0.5f;                  // continuous index
-    int k = __float2int_rd(__log2f(kSqrt5Pi * P.nf * omz2) * kInvLog2Phi2);
+    int k = __float2int_rd(__fmaf_rn(lg2_approx(omz2), kInvLog2Phi2, P.zone0));
     k = max(2, min(k, kFibN - 3));
-    int32_t F0 = kFib.F[k], F1 = kFib.F[k + 1];
-    float e0 = kFib.eps[k], e1 = kFib.eps[k + 1];
-    float sg = (k & 1) ? -1.0f : 1.0f;
-    float u = sg * __fmaf_rn(-(float)F1, t, e1 * ic);
-    float v = sg * __fmaf_rn((float)F0, t, -e0 * ic);
+    const float4 ab = *reinterpret_cast<const float4 *>(&kZones.z[k].au);
+    const int2 FF = *reinterpret_cast<const int2 *>(&kZones.z[k].F0);
+    const int32_t F0 = FF.x, F1 = FF.y;
+    float u = __fmaf_rn(ab.x, t, ab.y * ic);
+    float v = __fmaf_rn(ab.z, t, ab.w * ic);
     float ru = rintf(u), rv = rintf(v);
     bool pu = u >= ru, pv = v >= rv;
+    Corner c;
+    c.b = (int32_t)ru * F0 + (int32_t)rv * F1;
+    c.G0 = pu ? (pv ? F0 : -F1) : (pv ? F1 : -F0);
+    c.G1 = pu ? (pv ? F1 : F0) : (pv ? -F0 : -F1);
+    c.reach = F0 + F1;
+    return c;
+}
+
+__device__ __forceinline__ Source window_of(const PointSetK &P, const Corner &c)
+{
     Source s;
-    const int32_t base = (int32_t)ru * F0 + (int32_t)rv * F1;
-    s.G0 = pu ? (pv ? F0 : -F1) : (pv ? F1 : -F0);
-    s.G1 = pu ? (pv ? F1 : F0) : (pv ? -F0 : -F1);
-    s.b0 = base - s.G0 - s.G1;
-    const int32_t reach = 2 * (F0 + F1);
-    s.interior = (base - reach >= 0) && (base + reach < (int32_t)P.n);
+    s.G0 = c.G0;
+    s.G1 = c.G1;
+    s.b0 = c.b - c.G0 - c.G1;
+    s.interior = (c.b - 2 * c.reach >= 0) && (c.b + 2 * c.reach < (int32_t)P.n);
     s.scan_cnt = 0;
     s.bits = 4;
     return s;
@@ -455,11 +488,11 @@ constexpr int kWindow = 12;
 // Slot of window candidate j (0..11).
 __device__ __forceinline__ constexpr uint32_t slot5(int j) { return j < 11 ? (uint32_t)j : 14u; }
 
-// Candidate source of one query (see above).
-__device__ __forceinline__ Source candidate_source(const PointSetK &P, float3 qh)
+// Candidate source of one query (see above): `s` becomes a scan of all points or
+// of the 64 nearest a pole where one applies (true), else a window is needed.
+__device__ __forceinline__ bool scan_source(const PointSetK &P, float3 qh, Source &s)
 {
     const int32_t n = (int32_t)P.n;
-    Source s;
     s.b0 = 0;
     s.G0 = 1;
     s.G1 = 4;
@@ -467,16 +500,21 @@ __device__ __forceinline__ Source candidate_source(const PointSetK &P, float3 qh
     if (n <= 128) {
         s.scan_cnt = n;
         s.bits = 7;
-        return s;
+        return true;
     }
     float icn = (P.nf * (1.0f - qh.z) - 1.0f) * 0.5f;
     float ics = (P.nf * (1.0f + qh.z) - 1.0f) * 0.5f;
     s.scan_cnt = 64;
     s.bits = 6;
-    if (icn < 16.0f) return s;
+    if (icn < 16.0f) return true;
     s.b0 = n - 64;
-    if (ics < 16.0f) return s;
-    return lattice_window(P, qh);
+    return ics < 16.0f;
+}
+__device__ __forceinline__ Source candidate_source(const PointSetK &P, float3 qh)
+{
+    Source s;
+    if (scan_source(P, qh, s)) return s;
+    return window_of(P, lattice_corner(P, qh));
 }
 
 // Tier-1 squared distance from the hi parts only.
@@ -519,13 +557,10 @@ using Top5 = TopK<5>;
 // and run by one lane it holds its warp and CTA for tens of thousands of
 // cycles (FP64 division and square root alone take hundreds of cycles each on
 // this GPU).
-__device__ __forceinline__ Top5 knn5(const PointSetK &P, const SphereK &S, float3 h, uint32_t *status,
+__device__ __forceinline__ Top5 knn5(const PointSetK &P, float3 qh, float3 ql, const Source &src, uint32_t *status,
                                      bool &uncertain)
 {
-    float3 qh, ql;
-    unit_hit_df(S, h, qh, ql);
     const int32_t n = (int32_t)P.n;
-    const Source src = candidate_source(P, qh);
     const uint32_t mask1 = (1u << src.bits) - 1u;
     constexpr uint32_t kNone = 0xffffffffu;
 
@@ -932,12 +967,10 @@ static __device__ __noinline__ TopK<9> knn9_rerank(const PointSetK P, const Sphe
 
 // The 9 nearest points of the unit hit in (distance, index) order with their
 // double-float squared distances; cnt = min(9, n).
-__device__ __forceinline__ TopK<9> knn9(const PointSetK &P, const SphereK &S, float3 h, uint32_t *status)
+__device__ __forceinline__ TopK<9> knn9(const PointSetK &P, const SphereK &S, float3 h, float3 qh, float3 ql,
+                                        const Source &src, uint32_t *status)
 {
-    float3 qh, ql;
-    unit_hit_df(S, h, qh, ql);
     const int32_t n = (int32_t)P.n;
-    const Source src = candidate_source(P, qh);
     const int bits = src.scan_cnt ? src.bits : 5;
     const uint32_t mask1 = (1u << bits) - 1u;
     constexpr uint32_t kNone = 0xffffffffu;

@@ -40,6 +40,12 @@ struct ViewK {
     // (host FP64, rounded), and whether the eye is clearly outside S.
     float f0[3], c0, ff0, inv2w, inv2h;
     uint32_t outside;
+    float q[6];              // certain_miss: q0 + q1 x + q2 y + q3 x^2 + q4 x y + q5 y^2 < 0 at pixel (x, y)
+    // Pixels outside columns [sx0, sx1) or rows [sy0, sy1) certainly miss S
+    // (the screen bound of certain_miss, widened by two pixels).
+    uint32_t sx0, sx1, sy0, sy1;
+    // lt / tiles_x for any lt < 2^31 is (lt * div_m) >> div_s (64-bit product)
+    uint32_t div_m, div_s;
 };
 
 // Sphere S: FP32 centre and radius for the ray/sphere step, the centre as a
@@ -55,14 +61,24 @@ struct SphereK {
     uint32_t centred;        // O == (0, 0, 0)
 };
 
-// One SF point set: p_i as hi/lo float4 pairs (w unused), n, n as float and
-// the reciprocal kernel radius 1/sqrt(4*pi/n).
+// Entries of the xy cache before point 0 and after point n - 1: points far from
+// S, which a lattice corner outside the index range reads.
+constexpr int32_t kPointPad = 64;
+
+// One SF point set: p_i as hi/lo float4 pairs (w unused) and, for the searches
+// that need x and y only (z is linear in i), as one float4 (x_hi, y_hi, x_lo,
+// y_lo) at entry kPointPad + i; n, n as float, the kernel radius sigma = sqrt(4*pi/n) as its
+// reciprocal and square, and the z step 2/n as a hi/lo pair with its half 1/n.
 struct PointSetK {
     const float4 *hi;
     const float4 *lo;
+    const float4 *xy;
     uint32_t n;
     float nf;
     float inv_sigma;
+    float sigma2;
+    float zone0;             // log_{Phi^2}(sqrt5*pi*n), the set's part of the zone number
+    float zstep_h, zstep_l, zhalf;
 };
 
 // Argument checks and view set-up shared by the entry points (lf_abi.cu): a
@@ -72,6 +88,8 @@ lf_status check_launch(const lf_launch *c);
 lf_status check_views(const lf_view *views, uint32_t n);
 ViewK camera_of(const lf_view &w);                  // the camera only (no tiling, no miss constants)
 ViewK view_params(const lf_view &w, const lf_launch &L, double R, const double O[3]);
+// The set of n points with caches hi [n], lo [n], xy [n + 2 kPointPad].
+PointSetK point_set_of(const float4 *hi, const float4 *lo, const float4 *xy, uint32_t n);
 
 }  // namespace lfk
 
@@ -85,7 +103,7 @@ struct lf_table {
     const float *scales;             // [M] or NULL (F32)
     void *owned_texels;              // non-NULL if the library owns the copy
     float *owned_scales;
-    float4 *points;                  // [2M + 2N]: origins hi, lo, then directions hi, lo
+    float4 *points;                  // origins hi, lo, xy, then directions hi, lo, xy
     uint32_t *scratch;               // device words and the queue of deferred rays (layout: lf_kernels.h)
     lfk::SphereK sphere;
     lfk::PointSetK po, pd;

@@ -13,19 +13,19 @@ constexpr int kLargeViews = 64;    // batches are split into launches of <= 64 v
 constexpr int kMaxBlock = 256;     // threads per CTA (tile_w * tile_h)
 constexpr uint32_t kStripTiles = 4;
 
-// Device words of a table or of a no-allocation render: [0] status, [1] tile
-// queue, [2] finished render CTAs, [3] finished fixup CTAs, bytes 16..23 the
+// Device words of a table or of a no-allocation render: [0] status, [3] finished
+// fixup CTAs, bytes 16..23 the
 // count of queued rays; the queued rays follow at byte kWordsBytes.
 constexpr uint32_t kWordsBytes = 256;
 constexpr uint32_t kDeferCap = 1u << 18;         // queued rays a table holds per launch
 constexpr unsigned kFixupCtas = 304, kFixupThreads = 256;   // the fixup grid when the occupancy query fails
-constexpr uint32_t kFixupWarps = kFixupThreads / 32;
 
 struct RenderParamsBase {
     SphereK sphere;
     PointSetK po, pd;
     const void *texels;            // [M][N][Cs]
     const float *scales;           // [M] (F16 / E4M3)
+    uint64_t table_bytes;          // rows_valid * N texels
     uint32_t N;                    // texels per origin row
     uint32_t C;                    // output / gradient channels (3 or 4)
     float *out;                    // forward: [P][C] FP32, or binary16 when out_f16
@@ -34,7 +34,7 @@ struct RenderParamsBase {
     const int32_t *idx_in;         // backward: the forward's [P][2K] indices, or NULL (search again)
     const float *grad_out;         // backward: [P][C]
     float *grad;                   // backward: [M][N][C]
-    uint32_t *status, *queue, *done;
+    uint32_t *status;
     // Rays whose fast-path order was not certain: the render kernel queues
     // them here and the fixup kernel that follows it on the stream renders
     // them (more than defer_cap in one launch: the fixup renders every ray).
@@ -44,7 +44,7 @@ struct RenderParamsBase {
     uint32_t defer_cap;
     uint64_t total_pixels;             // pixels of all views of the launch
     uint32_t n_views, total_tiles;
-    uint32_t tile_w, tile_h, warp_w, order, persistent;
+    uint32_t tile_w, tile_h, warp_w, order;
     uint32_t tw_log, th_log, ww_log;   // log2 of tile_w, tile_h, warp_w
     uint32_t rows_stored;              // origin rows present (upper hemisphere), 0: all
     uint32_t rows_valid;               // rows of the table (M or rows_stored)
@@ -58,14 +58,19 @@ struct RenderParams : RenderParamsBase {
     ViewK views[MAXV];
 };
 
-cudaError_t launch_render_small(int kind, bool bwd, const RenderParams<kSmallViews> &p, unsigned grid,
-                                unsigned block, cudaStream_t st);
-cudaError_t launch_render_large(int kind, bool bwd, const RenderParams<kLargeViews> &p, unsigned grid,
-                                unsigned block, cudaStream_t st);
-int render_occupancy(int kind, bool bwd, bool large, bool nine, unsigned block);
+// lf_render.cu: the forward launch (and, where it may queue rays, the exact pass).
+cudaError_t launch_render(int kind, const RenderParams<kSmallViews> &p, unsigned grid, unsigned block, cudaStream_t st);
+cudaError_t launch_render(int kind, const RenderParams<kLargeViews> &p, unsigned grid, unsigned block, cudaStream_t st);
+// lf_backward.cu: the gradient scatter.
+cudaError_t launch_backward(const RenderParams<kSmallViews> &p, unsigned grid, unsigned block, cudaStream_t st);
+cudaError_t launch_backward(const RenderParams<kLargeViews> &p, unsigned grid, unsigned block, cudaStream_t st);
+// lf_fixup.cu: the exact pass over the rays a render or backward launch queued.
+cudaError_t launch_fixup(int kind, bool bwd, const RenderParams<kSmallViews> &p, cudaStream_t st);
+cudaError_t launch_fixup(int kind, bool bwd, const RenderParams<kLargeViews> &p, cudaStream_t st);
 
 // lf_table.cu
-cudaError_t launch_build_points(uint32_t n, float4 *hi, float4 *lo, cudaStream_t st);
+// The caches of a set's n points; xy may be NULL.
+cudaError_t launch_build_points(uint32_t n, float4 *hi, float4 *lo, float4 *xy, cudaStream_t st);
 cudaError_t launch_pad_codes(const void *src, uint32_t M, uint32_t N, int bytes, void *dst, cudaStream_t st);
 cudaError_t launch_quantize(const float *src, uint32_t M, uint32_t N, uint32_t C, int dtype, void *codes,
                             float *scales, cudaStream_t st);
@@ -137,6 +142,11 @@ cudaError_t launch_post_filter(const PostParams &p, cudaStream_t st);
 
 // Fills the conservative-miss constants of a view for sphere (R, O) (lf_abi.cu).
 void fill_view_miss_consts(ViewK &k, double R, const double O[3]);
+// Fills the coefficients of certain_miss, and the screen bound, of a view whose
+// miss constants are set (lf_abi.cu).
+void fill_certain_miss(ViewK &k);
+void fill_screen_bound(ViewK &k);
+uint64_t table_bytes_of(int kind, uint32_t rows, uint32_t N);
 
 // Host-side constants of sphere S (lf_abi.cu): FP32 radius and centre for the
 // ray/sphere step, the centre as a hi/lo float pair and in FP64, and for the

@@ -10,8 +10,8 @@
 // fixed size, g_lf_noalloc_scratch, which every GPU that loads the library
 // holds until the process exits.
 //
-// Layout of the array: the hi/lo point caches of both SF sets (M + N points,
-// 32 B each), then 256 B of words (status, tile queue, finished CTAs, the
+// Layout of the array: the point caches of both SF sets (M + N points, 48 B
+// each), then 256 B of words (status, finished CTAs, the
 // count of rays queued for the exact fixup pass), then the queue itself
 // (kNoAllocDeferCap entries of 8 B). Every call rebuilds the point caches and
 // clears the words on its stream, so the array only ever holds the last
@@ -30,11 +30,12 @@
 namespace {
 
 constexpr uint64_t kNoAllocMaxPoints = LF_NOALLOC_MAX_POINTS;     // M + N
+constexpr uint64_t kPointsFloat4 = 3 * kNoAllocMaxPoints + 4 * lfk::kPointPad;   // the point caches
 constexpr uint64_t kWordsFloat4 = lfk::kWordsBytes / 16;             // 256 B of words
 constexpr uint32_t kNoAllocDeferCap = LF_NOALLOC_MAX_DEFERRED;       // queued rays per launch
 constexpr uint64_t kQueueFloat4 = kNoAllocDeferCap / 2;              // 8 B per queued ray
 
-static __device__ __align__(256) float4 g_lf_noalloc_scratch[2 * kNoAllocMaxPoints + kWordsFloat4 + kQueueFloat4];
+static __device__ __align__(256) float4 g_lf_noalloc_scratch[kPointsFloat4 + kWordsFloat4 + kQueueFloat4];
 
 lf_status na_fail(lf_status s, const char *fmt, ...)
 {
@@ -63,7 +64,7 @@ lf_status scratch_address(float4 **out)
 }
 
 template <int MAXV>
-lf_status launch_views(const lfk::RenderParamsBase &base, const lf_launch &L, int kind, int sm_count,
+lf_status launch_views(const lfk::RenderParamsBase &base, const lf_launch &L, int kind,
                        const lf_view *views, uint32_t nv, const lf_table_desc *d, cudaStream_t st)
 {
     static thread_local lfk::RenderParams<MAXV> p;
@@ -80,20 +81,9 @@ lf_status launch_views(const lfk::RenderParamsBase &base, const lf_launch &L, in
     p.tile_prefix[nv] = (uint32_t)tiles;
     p.n_views = nv;
     p.total_tiles = (uint32_t)tiles;
-    unsigned block = L.tile_w * L.tile_h;
-    unsigned grid = (unsigned)tiles;
-    if (L.persistent) {
-        int per_sm = L.ctas_per_sm ? (int)L.ctas_per_sm
-                                   : lfk::render_occupancy(kind, false, MAXV != lfk::kSmallViews, false, block);
-        uint64_t g = (uint64_t)sm_count * (uint64_t)per_sm;
-        grid = (unsigned)(g < tiles ? g : tiles);
-    }
+    const unsigned block = L.tile_w * L.tile_h, grid = (unsigned)tiles;
     if (grid == 0) return LF_OK;
-    cudaError_t e;
-    if constexpr (MAXV == lfk::kSmallViews)
-        e = lfk::launch_render_small(kind, false, p, grid, block, st);
-    else
-        e = lfk::launch_render_large(kind, false, p, grid, block, st);
+    const cudaError_t e = lfk::launch_render(kind, p, grid, block, st);
     if (e != cudaSuccess) return na_fail(LF_ERR_CUDA, "render launch: %s", cudaGetErrorString(e));
     return LF_OK;
 }
@@ -136,30 +126,23 @@ lf_status lf_render_noalloc(const lf_table_desc *d, const void *radiance_dev, co
         L = *launch;
     }
 
-    int dev = -1;
-    cudaError_t e = cudaGetDevice(&dev);
-    if (e != cudaSuccess) return na_fail(LF_ERR_CUDA, "cudaGetDevice: %s", cudaGetErrorString(e));
     float4 *base = nullptr;
     s = scratch_address(&base);
     if (s != LF_OK) return s;
-    int sm_count = 0;
-    e = cudaDeviceGetAttribute(&sm_count, cudaDevAttrMultiProcessorCount, dev);
-    if (e != cudaSuccess || sm_count <= 0)
-        return na_fail(LF_ERR_CUDA, "SM count of device %d: %s", dev, cudaGetErrorString(e));
     cudaStream_t st = (cudaStream_t)stream;
-    float4 *po_hi = base, *po_lo = base + M, *pd_hi = base + 2 * (uint64_t)M, *pd_lo = pd_hi + N;
-    uint32_t *words = reinterpret_cast<uint32_t *>(base + 2 * kNoAllocMaxPoints);
-    e = cudaMemsetAsync(words, 0, kWordsFloat4 * sizeof(float4), st);
-    if (e == cudaSuccess) e = lfk::launch_build_points(M, po_hi, po_lo, st);
-    if (e == cudaSuccess) e = lfk::launch_build_points(N, pd_hi, pd_lo, st);
+    float4 *po = base, *pd = base + 3 * (uint64_t)M + 2 * lfk::kPointPad;
+    float4 *po_lo = po + M, *po_xy = po + 2 * (uint64_t)M, *pd_lo = pd + N, *pd_xy = pd + 2 * (uint64_t)N;
+    uint32_t *words = reinterpret_cast<uint32_t *>(base + kPointsFloat4);
+    cudaError_t e = cudaMemsetAsync(words, 0, kWordsFloat4 * sizeof(float4), st);
+    if (e == cudaSuccess) e = lfk::launch_build_points(M, po, po_lo, po_xy, st);
+    if (e == cudaSuccess) e = lfk::launch_build_points(N, pd, pd_lo, pd_xy, st);
     if (e != cudaSuccess) return na_fail(LF_ERR_CUDA, "scratch set-up: %s", cudaGetErrorString(e));
 
     lfk::RenderParamsBase b;
     memset(&b, 0, sizeof b);
     lfk::fill_sphere_consts(b.sphere, d->radius, d->center);
-    const double four_pi = 12.566370614359172953850573533118;
-    b.po = {po_hi, po_lo, M, (float)M, (float)(1.0 / std::sqrt(four_pi / (double)M))};
-    b.pd = {pd_hi, pd_lo, N, (float)N, (float)(1.0 / std::sqrt(four_pi / (double)N))};
+    b.po = lfk::point_set_of(po, po_lo, po_xy, M);
+    b.pd = lfk::point_set_of(pd, pd_lo, pd_xy, N);
     b.texels = radiance_dev;
     b.scales = quant ? row_scales_dev : nullptr;
     b.N = N;
@@ -167,17 +150,14 @@ lf_status lf_render_noalloc(const lf_table_desc *d, const void *radiance_dev, co
     b.out = out_dev;
     b.idx = idx_dev;
     b.status = words;
-    b.queue = words + 1;
-    b.done = words + 2;
     b.defer_done = words + 3;
     b.defer_count = reinterpret_cast<unsigned long long *>(words + 4);
-    b.defer_items = reinterpret_cast<unsigned long long *>(base + 2 * kNoAllocMaxPoints + kWordsFloat4);
+    b.defer_items = reinterpret_cast<unsigned long long *>(base + kPointsFloat4 + kWordsFloat4);
     b.defer_cap = kNoAllocDeferCap;
     b.tile_w = L.tile_w;
     b.tile_h = L.tile_h;
     b.warp_w = L.warp_w;
     b.order = L.order;
-    b.persistent = L.persistent;
     b.tw_log = (uint32_t)__builtin_ctz(L.tile_w);
     b.th_log = (uint32_t)__builtin_ctz(L.tile_h);
     b.ww_log = (uint32_t)__builtin_ctz(L.warp_w);
@@ -185,12 +165,13 @@ lf_status lf_render_noalloc(const lf_table_desc *d, const void *radiance_dev, co
     b.rows_valid = upper ? M / 2 : M;
     b.nearest_only = d->k_nearest == 1 ? 1u : 0u;
     b.rows_stored = upper ? M / 2 : 0u;
-    int kind = !quant ? (C == 4 ? lfk::kF32C4 : lfk::kF32C3) : (d->dtype == LF_DTYPE_F16 ? lfk::kF16C4 : lfk::kE4M3C4);
+    const int kind = !quant ? (C == 4 ? lfk::kF32C4 : lfk::kF32C3) : (d->dtype == LF_DTYPE_F16 ? lfk::kF16C4 : lfk::kE4M3C4);
+    b.table_bytes = lfk::table_bytes_of(kind, b.rows_valid, N);
     if (n_views <= (uint32_t)lfk::kSmallViews)
-        return launch_views<lfk::kSmallViews>(b, L, kind, sm_count, views, n_views, d, st);
+        return launch_views<lfk::kSmallViews>(b, L, kind, views, n_views, d, st);
     for (uint32_t v0 = 0; v0 < n_views; v0 += lfk::kLargeViews) {
         uint32_t nv = n_views - v0 < (uint32_t)lfk::kLargeViews ? n_views - v0 : (uint32_t)lfk::kLargeViews;
-        s = launch_views<lfk::kLargeViews>(b, L, kind, sm_count, views + v0, nv, d, st);
+        s = launch_views<lfk::kLargeViews>(b, L, kind, views + v0, nv, d, st);
         if (s != LF_OK) return s;
     }
     return LF_OK;
@@ -204,7 +185,7 @@ lf_status lf_noalloc_sync_status(void *stream)
     if (s != LF_OK) return s;
     cudaError_t e = cudaStreamSynchronize((cudaStream_t)stream);
     if (e != cudaSuccess) return na_fail(LF_ERR_CUDA, "stream synchronize: %s", cudaGetErrorString(e));
-    uint32_t *words = reinterpret_cast<uint32_t *>(base + 2 * kNoAllocMaxPoints);
+    uint32_t *words = reinterpret_cast<uint32_t *>(base + kPointsFloat4);
     uint32_t w = 0;
     e = cudaMemcpy(&w, words, sizeof w, cudaMemcpyDeviceToHost);
     if (e != cudaSuccess) return na_fail(LF_ERR_CUDA, "status read: %s", cudaGetErrorString(e));

@@ -1,0 +1,452 @@
+// lf_ray.cuh -- per-ray steps shared by the render, backward and fixup kernels:
+// tiles and pixels, the points within the kernel radius of a hit, nearest
+// sampling, the texel blend and the image and index stores.
+#pragma once
+
+#include <cuda_fp16.h>
+#include <cuda_runtime.h>
+
+#include "lf_device.cuh"
+#include "lf_kernels.h"
+
+namespace lfk {
+
+// ---------------------------------------------------------------------------
+// Tiles
+// ---------------------------------------------------------------------------
+// Tile t of the launch -> (view, tile column, tile row).
+__device__ __forceinline__ void tile_of(const RenderParamsBase &p, const ViewK *views, const uint32_t *prefix,
+                                        uint32_t nv, uint32_t t, uint32_t &v, uint32_t &tx, uint32_t &ty)
+{
+    uint32_t lo = 0, hi = nv;          // largest v with prefix[v] <= t
+    while (hi - lo > 1) {
+        uint32_t mid = (lo + hi) >> 1;
+        if (prefix[mid] <= t) lo = mid; else hi = mid;
+    }
+    v = lo;
+    const uint32_t lt = t - prefix[v], tiles_x = views[v].tiles_x;
+    if (p.order == 0) {
+        ty = (uint32_t)(((uint64_t)lt * views[v].div_m) >> views[v].div_s);     // lt / tiles_x
+        tx = lt - ty * tiles_x;
+    } else {                           // strips of kStripTiles tile rows, column by column
+        const uint32_t strip = lt / (tiles_x * kStripTiles);
+        const uint32_t r = lt - strip * tiles_x * kStripTiles;
+        const uint32_t hs = min(kStripTiles, views[v].tiles_y - strip * kStripTiles);
+        tx = r / hs;
+        ty = strip * kStripTiles + (r - tx * hs);
+    }
+}
+
+// Pixel of this thread in tile (tx, ty): tile and warp shapes are powers of
+// two, so the mapping is shifts and masks.
+__device__ __forceinline__ void pixel_of(const RenderParamsBase &p, uint32_t tx, uint32_t ty, uint32_t &px,
+                                         uint32_t &py)
+{
+    uint32_t warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    uint32_t wx_log = p.tw_log - p.ww_log;              // log2(warps per tile row)
+    px = (tx << p.tw_log) + ((warp & ((1u << wx_log) - 1u)) << p.ww_log) + (lane & ((1u << p.ww_log) - 1u));
+    py = (ty << p.th_log) + ((warp >> wx_log) << (5u - p.ww_log)) + (lane >> p.ww_log);
+}
+
+// True when no pixel of tile (tx, ty) can hit S: the tile lies outside the
+// view's screen bound of the rays that certain_miss keeps.
+__device__ __forceinline__ bool tile_misses(const RenderParamsBase &p, const ViewK &v, uint32_t tx, uint32_t ty)
+{
+    const uint32_t x0 = tx << p.tw_log, y0 = ty << p.th_log;
+    return x0 >= v.sx1 || x0 + p.tile_w <= v.sx0 || y0 >= v.sy1 || y0 + p.tile_h <= v.sy0;
+}
+
+__device__ __forceinline__ PointSetK point_set(const RenderParamsBase &p, int s)
+{
+    PointSetK P;
+    P.hi = s ? p.pd.hi : p.po.hi;
+    P.lo = s ? p.pd.lo : p.po.lo;
+    P.xy = s ? p.pd.xy : p.po.xy;
+    P.n = s ? p.pd.n : p.po.n;
+    P.nf = s ? p.pd.nf : p.po.nf;
+    P.inv_sigma = s ? p.pd.inv_sigma : p.po.inv_sigma;
+    P.sigma2 = s ? p.pd.sigma2 : p.po.sigma2;
+    P.zone0 = s ? p.pd.zone0 : p.po.zone0;
+    P.zstep_h = s ? p.pd.zstep_h : p.po.zstep_h;
+    P.zstep_l = s ? p.pd.zstep_l : p.po.zstep_l;
+    P.zhalf = s ? p.pd.zhalf : p.po.zhalf;
+    return P;
+}
+
+// Queues ray (view vi, pixel px, py) for the fixup kernel; bit s of pend marks
+// a set whose search was not certain, kPendImage that the image of the ray is
+// left to the fixup kernel too. When the queue is full the count still grows
+// past defer_cap, which tells the fixup kernel to take every ray.
+constexpr uint32_t kPendImage = 4u;
+__device__ __forceinline__ void defer_push(const RenderParamsBase &p, uint32_t vi, uint32_t px, uint32_t py,
+                                           uint32_t pend)
+{
+    const unsigned long long slot = atomicAdd(p.defer_count, 1ull);
+    if (slot < p.defer_cap)
+        p.defer_items[slot] = ((unsigned long long)pend << 48) | ((unsigned long long)vi << 32) |
+                              ((unsigned long long)py << 16) | px;
+}
+
+// ---------------------------------------------------------------------------
+// The neighbours of nonzero weight.
+//
+// The tent of radius sigma = sqrt(4 pi / n) (the square root of a point's share
+// of the sphere) gives weight 0 to every point at sigma or farther, and the
+// points nearer than sigma are always 1 to 5 and the nearest lies within 0.78
+// sigma (tests/test_kernel_radius.py: the 6th nearest is at least 1.04 sigma
+// away for every n, at the poles too). So the weighted neighbours among the 5
+// or 9 nearest are exactly the points within sigma, whatever their order: an
+// image needs no ranking, no certificate of an order and no exact pass. Away
+// from the poles those points lie among 7 corners of the lattice window in the
+// quadrant's turned basis (same test; lattice_corner has the other corners):
+//   (0,0) (0,1) (1,0) (1,1) (0,-1) (-1,1) (-1,0).
+// Ranking 12 corners with a 37-comparator network, the order certificate and
+// the double-float distances of the winners cost about 1,250 thread
+// instructions per hit ray more than testing 7 distances against sigma.
+//
+// A ray's two lists (at most kListSlots entries: point index, squared
+// distance) wait in shared memory, one column per thread.
+// ---------------------------------------------------------------------------
+constexpr int kListSlots = 5;
+struct RayLists {
+    uint2 e[2][kListSlots][kMaxBlock];
+};
+
+// q_z - z_c of the unit hit and SF point c (z_c = 1 - (2 c + 1) / n), to about
+// 2^-24 of itself: c * 2/n as an exact product sum, every cancelling step
+// exact.
+__device__ __forceinline__ float z_offset(const PointSetK &P, int32_t c, float qzh, float qzl)
+{
+    const float cf = __int2float_rn(c);                  // exact: c <= 2^24
+    const float t = __fmul_rn(cf, P.zstep_h);
+    const float e = __fadd_rn(__fmaf_rn(cf, P.zstep_h, -t), __fmaf_rn(cf, P.zstep_l, P.zhalf));
+    const df s = two_sum(t, -1.0f);
+    return __fadd_rn(__fadd_rn(qzh, s.h), __fadd_rn(__fadd_rn(qzl, s.l), e));
+}
+
+// Squared distance of the unit hit to point i (-kPointPad .. n + kPointPad - 1;
+// far outside [0, n)), with dz = q_z - z_i at hand.
+__device__ __forceinline__ float dist2_xy(const PointSetK &P, int32_t i, float3 qh, float3 ql, float dz,
+                                          uint32_t *status)
+{
+    const float4 a = __ldg(P.xy + LF_DINDEX((uint32_t)(i + kPointPad), P.n + 2 * kPointPad, status, kStatusDebugPoint));
+    const float dx = __fadd_rn(__fsub_rn(qh.x, a.x), __fsub_rn(ql.x, a.z));
+    const float dy = __fadd_rn(__fsub_rn(qh.y, a.y), __fsub_rn(ql.y, a.w));
+    return __fmaf_rn(dx, dx, __fmaf_rn(dy, dy, __fmul_rn(dz, dz)));
+}
+
+// Lists the points within sigma of the unit hit qh + ql in `list` (column of
+// this thread); their number (1 to 5). Sets of at most 128 points are scanned,
+// and within 8 continuous indices of a pole the 28 points nearest it (the 7
+// corners hold every point within sigma from 6 indices on, and no point within
+// sigma of such a hit has an index of 24 or more; tests/test_kernel_radius.py).
+// Corners past either end of the index range read the cache's padding, points
+// far from S. With RANK, `src` gets the candidate source of rank5 and `pre` the
+// squared distances of its 12 corners.
+template <bool RANK>
+__device__ __forceinline__ int points_within(const PointSetK &P, float3 qh, float3 ql, uint2 *list, uint32_t *status,
+                                             Source &src, float (&pre)[kWindow])
+{
+    const int32_t n = (int32_t)P.n;
+    uint2 *w = list;
+    const uint2 *const end = list + kListSlots * kMaxBlock;
+    int32_t scan0 = 0, scan_cnt = n;
+    if (n > 128) {
+        const float icn = (P.nf * (1.0f - qh.z) - 1.0f) * 0.5f, ics = (P.nf * (1.0f + qh.z) - 1.0f) * 0.5f;
+        scan_cnt = icn < 8.0f || ics < 8.0f ? 28 : 0;
+        scan0 = icn < 8.0f ? 0 : n - 28;
+    }
+    if (scan_cnt == 0) {
+        const Corner c = lattice_corner(P, qh);
+        if constexpr (RANK) {
+            if (!scan_source(P, qh, src)) src = window_of(P, c);
+        }
+        // never taken: keeps every access within the padded cache whatever the hit's values are
+        const int32_t reach = RANK ? 2 * c.reach : c.reach;
+        if (c.b - reach < -kPointPad || c.b + reach >= n + kPointPad) return 0;
+        const float zb = z_offset(P, c.b, qh.z, ql.z);
+        const float z0 = __fmul_rn(__int2float_rn(c.G0), P.zstep_h);
+        const float z1 = __fmul_rn(__int2float_rn(c.G1), P.zstep_h);
+        const float zp = __fadd_rn(zb, z0), zm = __fsub_rn(zb, z0);
+        const int32_t b = c.b, ip = b + c.G0, im = b - c.G0;
+        const int32_t idx[7] = {b, b + c.G1, ip, ip + c.G1, b - c.G1, im + c.G1, im};
+        const float dz[7] = {zb, __fadd_rn(zb, z1), zp, __fadd_rn(zp, z1), __fsub_rn(zb, z1), __fadd_rn(zm, z1), zm};
+        float d2[7];
+#pragma unroll
+        for (int j = 0; j < 7; ++j) d2[j] = dist2_xy(P, idx[j], qh, ql, dz[j], status);
+#pragma unroll
+        for (int j = 0; j < 7; ++j) {
+            if (d2[j] < P.sigma2 && (j < kListSlots || w < end)) {
+                *w = make_uint2((uint32_t)idx[j], __float_as_uint(d2[j]));
+                w += kMaxBlock;
+            }
+        }
+        if constexpr (RANK) {
+            constexpr int kSlot[7] = {5, 9, 6, 10, 1, 8, 4};
+#pragma unroll
+            for (int j = 0; j < 7; ++j) pre[kSlot[j]] = d2[j];
+            const float zpp = __fadd_rn(zp, z0);
+            const int32_t ix[5] = {im - c.G1, ip - c.G1, ip + c.G0 - c.G1, ip + c.G0, ip + 2 * c.G1};
+            const float dzx[5] = {__fsub_rn(zm, z1), __fsub_rn(zp, z1), __fsub_rn(zpp, z1), zpp,
+                                  __fadd_rn(__fadd_rn(zp, z1), z1)};
+            constexpr int kSlotX[5] = {0, 2, 3, 7, 11};      // slot 14 is window candidate 11
+#pragma unroll
+            for (int j = 0; j < 5; ++j) pre[kSlotX[j]] = dist2_xy(P, ix[j], qh, ql, dzx[j], status);
+        }
+    } else {
+        if constexpr (RANK) scan_source(P, qh, src);
+#pragma unroll 4
+        for (int j = 0; j < scan_cnt; ++j) {
+            const int32_t i = scan0 + j;
+            const float d2 = dist2_df(P, LF_DINDEX(i, P.n, status, kStatusDebugPoint), qh, ql);
+            if (d2 < P.sigma2 && w < end) {
+                *w = make_uint2((uint32_t)i, __float_as_uint(d2));
+                w += kMaxBlock;
+            }
+        }
+    }
+    return (int)(w - list) / kMaxBlock;
+}
+
+// The indices of the 5 nearest points in (distance, index) order, -1 past the
+// set's size; false when the FP32 distances cannot settle the order, which is
+// then left to the exact pass. `src`, `pre`: from points_within (corners outside
+// the index range are far, and at least five lie inside it). The distances are those of dist2_xy and dist2_df, whose error is below
+// e(d2) = 2^-19 sigma d + 2^-21 d2 (z differences off by at most 2^-20 sigma,
+// five roundings of the rest); the keys drop the low bits of a distance for the
+// slot. One bound, at the 6th key, serves all: with every one of the top 6 keys'
+// upper ends below the next key's lower end by more than 2 e and 2^-40 (far
+// above any FP64 rounding of the exact distances), the order and the membership
+// of the 5 are the exact ones, since every other key is at least the 6th. About
+// 0.2% of searches fail this. A first ranking by FP32 high parts alone (one
+// third of the arithmetic on 5 of the 12 corners) is certain less often and
+// needs a second, divergent one for 3% of the searches: 4% slower.
+__device__ __forceinline__ bool rank5(const PointSetK &P, float3 qh, float3 ql, const Source &src, uint32_t *status,
+                                      const float (&pre)[kWindow], int32_t (&ix)[5])
+{
+    constexpr uint32_t kNone = 0xffffffffu;
+    const uint32_t mask = (1u << src.bits) - 1u;
+    uint32_t k[12];
+    if (src.scan_cnt == 0) {
+#pragma unroll
+        for (int j = 0; j < kWindow; ++j) k[j] = (__float_as_uint(pre[j]) & ~15u) | slot5(j);
+        select7_of12(k);
+    } else {
+        uint32_t s7[7];
+#pragma unroll
+        for (int m = 0; m < 7; ++m) s7[m] = kNone;
+#pragma unroll 1
+        for (int j = 0; j < src.scan_cnt; ++j) {
+            const int32_t i = src.b0 + j;
+            const float d2 = dist2_df(P, LF_DINDEX(i, P.n, status, kStatusDebugPoint), qh, ql);
+            insert7(s7, (__float_as_uint(d2) & ~mask) | (uint32_t)j);
+        }
+#pragma unroll
+        for (int m = 0; m < 7; ++m) k[m] = s7[m];
+    }
+    const float d6 = fminf(__uint_as_float(k[5] | mask), 4.5f);   // an empty slot is all ones: 4.5 > any chord
+    const float e = __fmaf_rn(0x1p-21f, d6, 0x1p-19f * sqrt_approx(d6 * P.sigma2));
+    const float gap = __fmaf_rn(2.0f, e, 0x1p-40f);
+    bool sure = true;
+#pragma unroll
+    for (int m = 0; m < 5; ++m) {
+        sure &= (k[m + 1] == kNone) |
+                (__fsub_rn(__uint_as_float(k[m + 1] & ~mask), __uint_as_float(k[m] | mask)) > gap);
+        ix[m] = k[m] != kNone ? source_index(src, k[m] & mask) : -1;
+    }
+    return sure;
+}
+
+// Tent weight of a listed point.
+__device__ __forceinline__ float tent(float d2, float inv_sigma)
+{
+    return __saturatef(__fmaf_rn(-sqrt_approx(d2), inv_sigma, 1.0f));
+}
+
+// Nearest sampling: the list becomes its nearest entry, with distance 0
+// (weight 1). False when the second is too close for the FP32 distances to
+// tell: their error is at most 2^-20 sigma per component difference in z and
+// 2^-22 of the result otherwise, so 2^-19 sigma d + 2^-21 d^2; the gap asked
+// for is twice that and 2^-40.
+__device__ __forceinline__ bool nearest_listed(const PointSetK &P, uint2 *list, int c)
+{
+    float d1 = 8.0f, d2 = 8.0f;
+    uint32_t i1 = 0;
+#pragma unroll
+    for (int m = 0; m < kListSlots; ++m) {
+        const uint2 e = list[m * kMaxBlock];
+        const float d = m < c ? __uint_as_float(e.y) : 8.0f;
+        i1 = d < d1 ? e.x : i1;
+        d2 = fminf(d2, fmaxf(d, d1));
+        d1 = fminf(d1, d);
+    }
+    d2 = fminf(d2, P.sigma2);                            // a second point beyond the list is at sigma or farther
+    const float err = __fmaf_rn(0x1p-20f, d2, __fmaf_rn(0x1p-18f, sqrt_approx(d2 * P.sigma2), 0x1p-40f));
+    list[0] = make_uint2(i1, 0u);
+    return d2 - d1 > err;
+}
+
+// Upper-hemisphere tables: keeps the listed origins whose rows are stored.
+__device__ __forceinline__ int keep_stored(uint2 *list, int c, uint32_t rows)
+{
+    int k = 0;
+#pragma unroll 1
+    for (int m = 0; m < c; ++m) {
+        const uint2 e = list[m * kMaxBlock];
+        if (e.x < rows) list[kMaxBlock * k++] = e;
+    }
+    return k;
+}
+
+// Upper-hemisphere tables, a hit with no stored origin within sigma: if the
+// nearest stored origin is among the 5 nearest origins it takes weight 1, else
+// the ray is masked. Returns the number of listed points (1 or 0); sets
+// `uncertain` when the distances are too close to tell (nearest_listed's
+// bound, taken at 1.75 sigma, beyond which no 5th nearest lies).
+__device__ __forceinline__ int nearest_stored(const PointSetK &P, float3 qh, float3 ql, uint32_t rows, uint2 *list,
+                                              bool &uncertain)
+{
+    const float sigma = sqrtf(P.sigma2);
+    // row i is stored iff z_i > 0 (up to the middle row of an odd count, z = 0)
+    if (qh.z < -1.75f * sigma) return 0;
+    const Source src = candidate_source(P, qh);
+    const int total = src.scan_cnt ? src.scan_cnt : kWindow;
+    const float err = __fmaf_rn(0x1p-16f, P.sigma2, 0x1p-40f);
+    float best = 8.0f;
+    int32_t ib = 0;
+    for (int pass = 0, nearer = 0;; ++pass) {
+        // pass 0: the nearest stored origin; pass 1: how many others are nearer
+#pragma unroll 1
+        for (int j = 0; j < total; ++j) {
+            const int32_t i = source_index(src, src.scan_cnt ? (uint32_t)j : slot5(j));
+            if ((uint32_t)i >= P.n) continue;
+            const float d2 = dist2_df(P, i, qh, ql);
+            if (pass == 0) {
+                if ((uint32_t)i < rows && d2 < best) {
+                    best = d2;
+                    ib = i;
+                }
+            } else if (i != ib) {
+                nearer += d2 < best ? 1 : 0;
+                uncertain |= fabsf(d2 - best) <= err;
+            }
+        }
+        if (pass == 0) {
+            if (best > 4.5f) return 0;                   // no stored origin in the window
+        } else {
+            if (nearer >= 5) return 0;
+            list[0] = make_uint2((uint32_t)ib, 0u);
+            return 1;
+        }
+    }
+}
+
+// ---------------------------------------------------------------------------
+// Blend and stores
+// ---------------------------------------------------------------------------
+// Packed FP32 pair FMA (one instruction for two lanes of a texel).
+__device__ __forceinline__ float2 ffma2(float2 a, float2 b, float2 c)
+{
+    unsigned long long ra = *reinterpret_cast<unsigned long long *>(&a);
+    unsigned long long rb = *reinterpret_cast<unsigned long long *>(&b);
+    unsigned long long rc = *reinterpret_cast<unsigned long long *>(&c);
+    unsigned long long rd;
+    asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(rd) : "l"(ra), "l"(rb), "l"(rc));
+    return *reinterpret_cast<float2 *>(&rd);
+}
+
+// binary16 image: the FP32 result rounded once (half the bytes to read back).
+__device__ __forceinline__ void store_f16(float *out, uint32_t C, uint64_t pix, float4 acc)
+{
+    const __half2 xy = __floats2half2_rn(acc.x, acc.y), zw = __floats2half2_rn(acc.z, acc.w);
+    if (C == 4) {
+        uint2 v;
+        v.x = *reinterpret_cast<const uint32_t *>(&xy);
+        v.y = *reinterpret_cast<const uint32_t *>(&zw);
+        __stcs(reinterpret_cast<uint2 *>(out) + pix, v);
+    } else {
+        unsigned short *o = reinterpret_cast<unsigned short *>(out) + pix * 3;
+        __stcs(o, __half_as_ushort(__low2half(xy)));
+        __stcs(o + 1, __half_as_ushort(__high2half(xy)));
+        __stcs(o + 2, __half_as_ushort(__low2half(zw)));
+    }
+}
+
+__device__ __forceinline__ uint64_t pixel_index(const ViewK &v, uint32_t px, uint32_t py)
+{
+    return v.out_offset + (uint64_t)py * v.width + px;
+}
+
+__device__ __forceinline__ void store_image(const RenderParamsBase &p, uint64_t pix, float4 acc)
+{
+    if (p.out_f16) {
+        store_f16(p.out, p.C, pix, acc);
+    } else if (p.C == 4) {
+        __stcs(reinterpret_cast<float4 *>(p.out) + pix, acc);
+    } else {
+        float *o = p.out + pix * 3;
+        __stcs(o, acc.x);
+        __stcs(o + 1, acc.y);
+        __stcs(o + 2, acc.z);
+    }
+}
+
+// The K origin and K direction indices of one ray.
+template <int K>
+__device__ __forceinline__ void store_idx(const RenderParamsBase &p, uint64_t pix, const int32_t (&io)[K],
+                                          const int32_t (&jd)[K])
+{
+    int2 *q = reinterpret_cast<int2 *>(p.idx + pix * (2 * K));
+    int32_t v[2 * K];
+#pragma unroll
+    for (int m = 0; m < K; ++m) {
+        v[m] = io[m];
+        v[K + m] = jd[m];
+    }
+#pragma unroll
+    for (int m = 0; m < K; ++m) q[m] = make_int2(v[2 * m], v[2 * m + 1]);
+}
+
+// Weights of one set's neighbours r (set 0: origins, 1: directions) by the
+// sampling mode; false when the ray is masked (an upper-hemisphere table with
+// no stored origin neighbour).
+template <int K>
+__device__ __forceinline__ bool set_weights(const RenderParamsBase &p, int s, float inv_sigma, TopK<K> &r,
+                                            float (&w)[K])
+{
+    if (p.nearest_only) {
+        // nearest sampling: the nearest point alone (Section 2, Fig. 2)
+        if (s == 0 && p.rows_stored && (uint32_t)r.i[0] >= p.rows_stored) return false;
+#pragma unroll
+        for (int m = 0; m < K; ++m) w[m] = m == 0 ? 1.0f : 0.0f;
+#pragma unroll
+        for (int m = 1; m < K; ++m) r.i[m] = -1;
+        return true;
+    }
+    if (s == 0 && p.rows_stored) return tent_weights_kept(r.d2, r.i, r.cnt, inv_sigma, p.rows_stored, w);
+    tent_weights(r.d2, r.cnt, inv_sigma, w);
+    return true;
+}
+
+__device__ __forceinline__ void add_to_grad(const RenderParamsBase &p, uint64_t key, float4 sum)
+{
+    key = LF_DINDEX(key, (uint64_t)p.rows_valid * p.N, p.status, kStatusDebugGrad);
+    if (p.C == 4) {
+        atomicAdd(reinterpret_cast<float4 *>(p.grad) + key, sum);
+    } else {
+        float *q = p.grad + key * 3;
+        atomicAdd(q, sum.x);
+        atomicAdd(q + 1, sum.y);
+        atomicAdd(q + 2, sum.z);
+    }
+}
+
+// dL/d(image) of pixel pix.
+__device__ __forceinline__ float4 grad_of(const RenderParamsBase &p, uint64_t pix)
+{
+    if (p.C == 4) return __ldg(reinterpret_cast<const float4 *>(p.grad_out) + pix);
+    const float *q = p.grad_out + pix * 3;
+    return make_float4(__ldg(q), __ldg(q + 1), __ldg(q + 2), 0.f);
+}
+
+}  // namespace lfk

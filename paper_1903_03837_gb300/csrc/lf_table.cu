@@ -17,10 +17,13 @@ constexpr double kTwoPi = 6.283185307179586476925286766559;
 // SF point p_i of a set of n points (Section 2, SF point set equation):
 // phi_i = 2*pi*frac(i/Phi) (phase truncated to 53 bits), z_i = 1 - (2i+1)/n,
 // p_i = (cos(phi_i) sin(theta_i), sin(phi_i) sin(theta_i), z_i) with
-// sin(theta_i) = sqrt((1 - z_i)(1 + z_i)); FP64, stored as hi/lo floats.
-__global__ void build_points_kernel(uint32_t n, float4 *hi, float4 *lo)
+// sin(theta_i) = sqrt((1 - z_i)(1 + z_i)); FP64, stored as hi/lo floats and,
+// when xy is given, as (x_hi, y_hi, x_lo, y_lo) between kPointPad far points on
+// either side.
+__global__ void build_points_kernel(uint32_t n, float4 *hi, float4 *lo, float4 *xy)
 {
     uint32_t i = blockIdx.x * blockDim.x + threadIdx.x;
+    if (xy && i < 2u * kPointPad) xy[i < (uint32_t)kPointPad ? i : n + i] = make_float4(4.0f, 4.0f, 0.0f, 0.0f);
     if (i >= n) return;
     uint64_t ii = i;
     uint64_t top = ii * kGoldHi + __umul64hi(ii, kGoldLo);
@@ -39,11 +42,12 @@ __global__ void build_points_kernel(uint32_t n, float4 *hi, float4 *lo)
     }
     hi[i] = make_float4(h[0], h[1], h[2], 0.0f);
     lo[i] = make_float4(l[0], l[1], l[2], 0.0f);
+    if (xy) xy[kPointPad + i] = make_float4(h[0], h[1], l[0], l[1]);
 }
 
-cudaError_t launch_build_points(uint32_t n, float4 *hi, float4 *lo, cudaStream_t st)
+cudaError_t launch_build_points(uint32_t n, float4 *hi, float4 *lo, float4 *xy, cudaStream_t st)
 {
-    build_points_kernel<<<(n + 255) / 256, 256, 0, st>>>(n, hi, lo);
+    build_points_kernel<<<(n + 255) / 256, 256, 0, st>>>(n, hi, lo, xy);   // at least 2 kPointPad threads
     return cudaGetLastError();
 }
 
