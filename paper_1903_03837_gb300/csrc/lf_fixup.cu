@@ -118,6 +118,7 @@ __device__ __forceinline__ void exact_ray(const RenderParamsBase &p, const ViewK
 template <int DT, int MAXV, bool BWD>
 __global__ void __launch_bounds__(kFixupThreads) fixup_kernel(const __grid_constant__ RenderParams<MAXV> p)
 {
+    __shared__ uint2 lists[BWD ? kFixupThreads / 32 : 1][BWD ? 2 * kListSlots : 1][32];
     const unsigned long long queued = *reinterpret_cast<volatile unsigned long long *>(p.defer_count);
     const bool all = queued > p.defer_cap;
     const unsigned long long total = all ? p.total_pixels : queued;
@@ -138,6 +139,20 @@ __global__ void __launch_bounds__(kFixupThreads) fixup_kernel(const __grid_const
             }
             py = (uint32_t)(r / p.views[vi].width);
             px = (uint32_t)(r - (unsigned long long)py * p.views[vi].width);
+        }
+        if constexpr (BWD) {
+            // the backward kernel has scattered the rays it did not queue: the same
+            // search (the same bits, in every lane alike) tells them apart
+            if (all) {
+                const ViewK &v = p.views[vi];
+                int co, cd;
+                int32_t io[1], jd[1];
+                pend = 0;
+                if (!certain_miss(v, px, py))
+                    ray_lists<0, 32>(p, v, camera_dir(v, px, py), &lists[threadIdx.x >> 5][0][threadIdx.x & 31u], co, cd,
+                                     io, jd, pend);
+                if (pend == 0) continue;
+            }
         }
         exact_ray<DT, BWD>(p, p.views[vi], px, py, pend);
     }

@@ -68,7 +68,7 @@ constexpr int32_t kPointPad = 64;
 // One SF point set: p_i as hi/lo float4 pairs (w unused) and, for the searches
 // that need x and y only (z is linear in i), as one float4 (x_hi, y_hi, x_lo,
 // y_lo) at entry kPointPad + i; n, n as float, the kernel radius sigma = sqrt(4*pi/n) as its
-// reciprocal and square, and the z step 2/n as a hi/lo pair with its half 1/n.
+// reciprocal and square (less 2^-20 of it), and the z step 2/n as a hi/lo pair with its half 1/n.
 struct PointSetK {
     const float4 *hi;
     const float4 *lo;

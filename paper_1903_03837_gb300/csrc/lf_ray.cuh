@@ -105,12 +105,10 @@ __device__ __forceinline__ void defer_push(const RenderParamsBase &p, uint32_t v
 // instructions per hit ray more than testing 7 distances against sigma.
 //
 // A ray's two lists (at most kListSlots entries: point index, squared
-// distance) wait in shared memory, one column per thread.
+// distance) wait in shared memory, one column per thread (STRIDE entries from one
+// slot to the next).
 // ---------------------------------------------------------------------------
 constexpr int kListSlots = 5;
-struct RayLists {
-    uint2 e[2][kListSlots][kMaxBlock];
-};
 
 // q_z - z_c of the unit hit and SF point c (z_c = 1 - (2 c + 1) / n), to about
 // 2^-24 of itself: c * 2/n as an exact product sum, every cancelling step
@@ -143,13 +141,13 @@ __device__ __forceinline__ float dist2_xy(const PointSetK &P, int32_t i, float3 
 // Corners past either end of the index range read the cache's padding, points
 // far from S. With RANK, `src` gets the candidate source of rank5 and `pre` the
 // squared distances of its 12 corners.
-template <bool RANK>
+template <bool RANK, int STRIDE>
 __device__ __forceinline__ int points_within(const PointSetK &P, float3 qh, float3 ql, uint2 *list, uint32_t *status,
                                              Source &src, float (&pre)[kWindow])
 {
     const int32_t n = (int32_t)P.n;
     uint2 *w = list;
-    const uint2 *const end = list + kListSlots * kMaxBlock;
+    const uint2 *const end = list + kListSlots * STRIDE;
     int32_t scan0 = 0, scan_cnt = n;
     if (n > 128) {
         const float icn = (P.nf * (1.0f - qh.z) - 1.0f) * 0.5f, ics = (P.nf * (1.0f + qh.z) - 1.0f) * 0.5f;
@@ -178,7 +176,7 @@ __device__ __forceinline__ int points_within(const PointSetK &P, float3 qh, floa
         for (int j = 0; j < 7; ++j) {
             if (d2[j] < P.sigma2 && (j < kListSlots || w < end)) {
                 *w = make_uint2((uint32_t)idx[j], __float_as_uint(d2[j]));
-                w += kMaxBlock;
+                w += STRIDE;
             }
         }
         if constexpr (RANK) {
@@ -201,11 +199,11 @@ __device__ __forceinline__ int points_within(const PointSetK &P, float3 qh, floa
             const float d2 = dist2_df(P, LF_DINDEX(i, P.n, status, kStatusDebugPoint), qh, ql);
             if (d2 < P.sigma2 && w < end) {
                 *w = make_uint2((uint32_t)i, __float_as_uint(d2));
-                w += kMaxBlock;
+                w += STRIDE;
             }
         }
     }
-    return (int)(w - list) / kMaxBlock;
+    return (int)(w - list) / STRIDE;
 }
 
 // The indices of the 5 nearest points in (distance, index) order, -1 past the
@@ -268,13 +266,14 @@ __device__ __forceinline__ float tent(float d2, float inv_sigma)
 // tell: their error is at most 2^-20 sigma per component difference in z and
 // 2^-22 of the result otherwise, so 2^-19 sigma d + 2^-21 d^2; the gap asked
 // for is twice that and 2^-40.
+template <int STRIDE>
 __device__ __forceinline__ bool nearest_listed(const PointSetK &P, uint2 *list, int c)
 {
     float d1 = 8.0f, d2 = 8.0f;
     uint32_t i1 = 0;
 #pragma unroll
     for (int m = 0; m < kListSlots; ++m) {
-        const uint2 e = list[m * kMaxBlock];
+        const uint2 e = list[m * STRIDE];
         const float d = m < c ? __uint_as_float(e.y) : 8.0f;
         i1 = d < d1 ? e.x : i1;
         d2 = fminf(d2, fmaxf(d, d1));
@@ -287,13 +286,14 @@ __device__ __forceinline__ bool nearest_listed(const PointSetK &P, uint2 *list, 
 }
 
 // Upper-hemisphere tables: keeps the listed origins whose rows are stored.
+template <int STRIDE>
 __device__ __forceinline__ int keep_stored(uint2 *list, int c, uint32_t rows)
 {
     int k = 0;
 #pragma unroll 1
     for (int m = 0; m < c; ++m) {
-        const uint2 e = list[m * kMaxBlock];
-        if (e.x < rows) list[kMaxBlock * k++] = e;
+        const uint2 e = list[m * STRIDE];
+        if (e.x < rows) list[STRIDE * k++] = e;
     }
     return k;
 }
@@ -339,6 +339,83 @@ __device__ __forceinline__ int nearest_stored(const PointSetK &P, float3 qh, flo
             return 1;
         }
     }
+}
+
+// Hits and lists of one ray of unit direction d; with IDX (5 or 9) also the
+// indices of its nearest points in (distance, index) order. False for a miss or
+// a masked ray. Bits of `pend`: defer_push. `lists`: this thread's column of the
+// origin list, the direction list after it.
+template <int IDX, int STRIDE>
+__device__ __forceinline__ bool ray_lists(const RenderParamsBase &p, const ViewK &v, float3 d, uint2 *lists, int &co,
+                                          int &cd, int32_t (&io)[IDX ? IDX : 1], int32_t (&jd)[IDX ? IDX : 1],
+                                          uint32_t &pend)
+{
+    __shared__ int s_stash[IDX ? IDX * kMaxBlock : 1];   // the origins' indices during the second search
+    float3 ho, hd;
+    if (!intersect_sphere(p.sphere, v.eye, d, ho, hd)) return false;
+    // One copy of the search serves both sets (instruction-cache footprint).
+#pragma unroll 1
+    for (int s = 0; s < 2; ++s) {
+        const PointSetK P = point_set(p, s);
+        uint2 *list = lists + s * kListSlots * STRIDE;
+        float3 qh, ql;
+        unit_hit_df(p.sphere, s ? hd : ho, qh, ql);
+        Source src;
+        float pre[kWindow];
+        int c = points_within<IDX == 5, STRIDE>(P, qh, ql, list, p.status, src, pre);
+        int32_t ix[IDX ? IDX : 1];
+        if constexpr (IDX == 5) {
+            if (!rank5(P, qh, ql, src, p.status, pre, ix)) pend |= 1u << s;
+        } else if constexpr (IDX == 9) {
+            const TopK<9> r = knn9(P, p.sphere, s ? hd : ho, qh, ql, candidate_source(P, qh), p.status);
+#pragma unroll
+            for (int m = 0; m < 9; ++m) ix[m] = r.i[m];
+        }
+        if (p.nearest_only) {
+            if (!nearest_listed<STRIDE>(P, list, c)) pend |= (1u << s) | kPendImage;
+            c = s == 0 && list[0].x >= p.rows_valid ? 0 : 1;
+        } else if (s == 0 && p.rows_stored) {
+            c = keep_stored<STRIDE>(list, c, p.rows_stored);
+            if (c == 0) {
+                // no stored origin within sigma: the nearest stored one of the 5 (9) nearest, if any
+                if constexpr (IDX == 9) {
+#pragma unroll
+                    for (int m = 8; m >= 0; --m)
+                        if ((uint32_t)ix[m] < p.rows_stored) {
+                            list[0] = make_uint2((uint32_t)ix[m], 0u);
+                            c = 1;
+                        }
+                } else {
+                    bool unc = false;
+                    c = nearest_stored(P, qh, ql, p.rows_stored, list, unc);
+                    if (unc) pend |= 1u | kPendImage;
+                }
+            }
+        }
+        if (pend & kPendImage) return true;              // the fixup kernel renders this ray
+        if (c == 0) {
+            pend = 0;
+            return false;
+        }
+        if (s == 0) {
+            co = c;
+            if constexpr (IDX != 0) {
+#pragma unroll
+                for (int m = 0; m < IDX; ++m) s_stash[m * kMaxBlock + threadIdx.x] = ix[m];
+            }
+        } else {
+            cd = c;
+            if constexpr (IDX != 0) {
+#pragma unroll
+                for (int m = 0; m < IDX; ++m) jd[m] = ix[m];
+            }
+        }
+    }
+    if constexpr (IDX != 0) {
+#pragma unroll
+        for (int m = 0; m < IDX; ++m) io[m] = s_stash[m * kMaxBlock + threadIdx.x];
+    }
+    return true;
 }
 
 // ---------------------------------------------------------------------------
@@ -434,10 +511,11 @@ __device__ __forceinline__ void add_to_grad(const RenderParamsBase &p, uint64_t 
     if (p.C == 4) {
         atomicAdd(reinterpret_cast<float4 *>(p.grad) + key, sum);
     } else {
+        // 12 bytes: the 8-byte-aligned pair of the three floats, and the third
         float *q = p.grad + key * 3;
-        atomicAdd(q, sum.x);
-        atomicAdd(q + 1, sum.y);
-        atomicAdd(q + 2, sum.z);
+        const bool odd = (reinterpret_cast<uintptr_t>(q) & 4u) != 0;
+        atomicAdd(reinterpret_cast<float2 *>(q + (odd ? 1 : 0)), odd ? make_float2(sum.y, sum.z) : make_float2(sum.x, sum.y));
+        atomicAdd(q + (odd ? 0 : 2), odd ? sum.x : sum.z);
     }
 }
 

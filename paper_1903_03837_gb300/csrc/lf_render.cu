@@ -59,81 +59,9 @@ __device__ __forceinline__ float4 texel_at(const RenderParamsBase &p, Off off)
     }
 }
 
-// Hits and lists of one ray of unit direction d; with IDX (5 or 9) also the
-// indices of its nearest points in (distance, index) order. False for a miss or
-// a masked ray. Bits of `pend`: defer_push.
-template <int IDX>
-__device__ __forceinline__ bool ray_lists(const RenderParamsBase &p, const ViewK &v, float3 d, RayLists &L, int &co,
-                                          int &cd, int32_t (&io)[IDX ? IDX : 1], int32_t (&jd)[IDX ? IDX : 1],
-                                          uint32_t &pend)
-{
-    __shared__ int s_stash[IDX ? IDX * kMaxBlock : 1];   // the origins' indices during the second search
-    float3 ho, hd;
-    if (!intersect_sphere(p.sphere, v.eye, d, ho, hd)) return false;
-    // One copy of the search serves both sets (instruction-cache footprint).
-#pragma unroll 1
-    for (int s = 0; s < 2; ++s) {
-        const PointSetK P = point_set(p, s);
-        uint2 *list = &L.e[s][0][threadIdx.x];
-        float3 qh, ql;
-        unit_hit_df(p.sphere, s ? hd : ho, qh, ql);
-        Source src;
-        float pre[kWindow];
-        int c = points_within<IDX == 5>(P, qh, ql, list, p.status, src, pre);
-        int32_t ix[IDX ? IDX : 1];
-        if constexpr (IDX == 5) {
-            if (!rank5(P, qh, ql, src, p.status, pre, ix)) pend |= 1u << s;
-        } else if constexpr (IDX == 9) {
-            const TopK<9> r = knn9(P, p.sphere, s ? hd : ho, qh, ql, candidate_source(P, qh), p.status);
-#pragma unroll
-            for (int m = 0; m < 9; ++m) ix[m] = r.i[m];
-        }
-        if (p.nearest_only) {
-            if (!nearest_listed(P, list, c)) pend |= (1u << s) | kPendImage;
-            c = s == 0 && list[0].x >= p.rows_valid ? 0 : 1;
-        } else if (s == 0 && p.rows_stored) {
-            c = keep_stored(list, c, p.rows_stored);
-            if (c == 0) {
-                // no stored origin within sigma: the nearest stored one of the 5 (9) nearest, if any
-                if constexpr (IDX == 9) {
-#pragma unroll
-                    for (int m = 8; m >= 0; --m)
-                        if ((uint32_t)ix[m] < p.rows_stored) {
-                            list[0] = make_uint2((uint32_t)ix[m], 0u);
-                            c = 1;
-                        }
-                } else {
-                    bool unc = false;
-                    c = nearest_stored(P, qh, ql, p.rows_stored, list, unc);
-                    if (unc) pend |= 1u | kPendImage;
-                }
-            }
-        }
-        if (pend & kPendImage) return true;              // the fixup kernel renders this ray
-        if (c == 0) {
-            pend = 0;
-            return false;
-        }
-        if (s == 0) {
-            co = c;
-            if constexpr (IDX != 0) {
-#pragma unroll
-                for (int m = 0; m < IDX; ++m) s_stash[m * kMaxBlock + threadIdx.x] = ix[m];
-            }
-        } else {
-            cd = c;
-            if constexpr (IDX != 0) {
-#pragma unroll
-                for (int m = 0; m < IDX; ++m) jd[m] = ix[m];
-            }
-        }
-    }
-    if constexpr (IDX != 0) {
-#pragma unroll
-        for (int m = 0; m < IDX; ++m) io[m] = s_stash[m * kMaxBlock + threadIdx.x];
-    }
-    return true;
-}
+struct RayLists {
+    uint2 e[2][kListSlots][kMaxBlock];
+};
 
 // Blend of one ray's listed origins and directions: sum of w_a w_b texel / (sum
 // w_a)(sum w_b). The loop over origins runs to the longest list of the warp and
@@ -198,7 +126,7 @@ __device__ __forceinline__ void render_ray(const RenderParamsBase &p, const View
     int co = 0, cd = 0;
     uint32_t pend = 0;
     bool hit = active && !certain_miss(v, px, py) &&
-               ray_lists<IDX>(p, v, camera_dir(v, px, py), L, co, cd, io, jd, pend);
+               ray_lists<IDX, kMaxBlock>(p, v, camera_dir(v, px, py), &L.e[0][0][threadIdx.x], co, cd, io, jd, pend);
     if (!hit || (pend & kPendImage)) co = cd = 0;
     const float4 acc = blend<DT, Off>(p, L, co, cd);
     if (!active) return;

@@ -4,8 +4,8 @@ current CUDA stream; the kernels of liblumipath.so do all of the work.
 * ``LightField``: a table on the GPU (create / render, FP32 or binary16 image /
   backward, searching again or from the forward's indices / launch shape)
 * ``RenderFunction``: ``torch.autograd.Function`` whose backward is the
-  library's scatter-add kernel, fed with the forward's indices (for fitting a
-  table to target views); ``fit_step``: one data-parallel fitting step
+  library's scatter-add kernel (for fitting a table to target views);
+  ``fit_step``: one data-parallel fitting step
 * ``precompute_table``: the light-field precompute of Section 2 (rays r_k with
   jittered origins through an analytic volume), on the GPU; ``render_volume``:
   the direct render of that volume along each pixel's ray (ground truth)
@@ -156,8 +156,10 @@ class RenderFunction(torch.autograd.Function):
     @staticmethod
     def forward(ctx, table: torch.Tensor, lf: LightField, views):
         ctx.lf, ctx.views = lf, views
-        out, idx = lf.render(views, with_idx=True)      # the backward reuses the indices
-        ctx.idx = idx
+        # five and nine neighbours: the image needs no ranking, and the backward's own
+        # unranked search costs less than writing and reading the indices; nearest
+        # sampling has them at hand
+        out, ctx.idx = lf.render(views, with_idx=lf.K == 1)
         return out
 
     @staticmethod
