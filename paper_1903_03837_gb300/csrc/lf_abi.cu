@@ -755,10 +755,8 @@ lf_status lf_render_volume(const lf_precompute_desc *d, const lf_blob *blobs, co
     lfk::SphereK S{};
     lfk::fill_sphere_consts(S, d->radius, d->center);
     cudaStream_t st = (cudaStream_t)stream;
-    for (uint32_t v = 0; v < n_views; ++v) {
-        cudaError_t e = lfk::launch_volume_direct(P, lfk::camera_of(views[v]), S, d->radius, st);
-        if (e != cudaSuccess) return cuda_fail(e, "direct volume render");
-    }
+    const cudaError_t e = lfk::launch_volume_direct(P, views, n_views, S, d->radius, d->center, st);
+    if (e != cudaSuccess) return cuda_fail(e, "direct volume render");
     return LF_OK;
 }
 

@@ -109,11 +109,12 @@ struct PrecomputeParams {
     float4 blob_col[kMaxBlobs];    // emit rgb, a_b = sqrt(log2(e) / 2) / s_b
 };
 cudaError_t launch_precompute(const PrecomputeParams &p, cudaStream_t st);
-// Direct render of the precompute's volume along the pixel rays of one view
-// (out at the view's out_offset; p.out, p.C and the volume fields are used;
-// R is the radius in FP64 for the far end of each ray).
-cudaError_t launch_volume_direct(const PrecomputeParams &p, const ViewK &v, const SphereK &S, double R,
-                                 cudaStream_t st);
+// Direct render of the precompute's volume along the pixel rays of n views (out
+// at each view's out_offset; p.out, p.C and the volume fields are used), one
+// launch per kVolumeViews views.
+constexpr int kVolumeViews = 32;
+cudaError_t launch_volume_direct(const PrecomputeParams &p, const lf_view *views, uint32_t n, const SphereK &S, double R,
+                                 const double O[3], cudaStream_t st);
 
 // lf_post.cu: the learned post-filter of the light-field image. Weights in
 // framework (OIHW) order, FP32: W1 [16][4][3][3], b1 [16], W2 [16][16][3][3],

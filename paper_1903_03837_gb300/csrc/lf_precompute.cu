@@ -9,8 +9,9 @@
 // b at step k (t_k = (k + 1/2) dt) is
 //   exp2(la_b - y_k^2),  la_b = log2(kappa_b) - a_b^2 |f_b x d|^2,
 //                        y_k  = a_b (f_b . d + 1/2 dt) + k (a_b dt),
-// two fma and one ex2 per blob-step (with blobs taken in pairs: one packed
-// fma, mul and sub per pair and two ex2). The cross product keeps the distance of
+// two fma and one ex2 per blob-step (blobs in pairs: two packed fma and two ex2 a
+// pair, the exponent as y_k^2 - la_b with its sign flipped on the way into ex2).
+// The cross product keeps the distance of
 // the ray from a narrow blob's centre accurate (|f|^2 - (f.d)^2 would cancel).
 // The emission is accumulated per blob, G_b += w_k g_bk with w_k the step's
 // compositing weight, and turned into colour once per sample: sum_b G_b emit_b
@@ -44,18 +45,6 @@ __device__ __forceinline__ float2 fma2(float2 a, float2 b, float2 c)
     asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(d) : "l"(pk(a)), "l"(pk(b)), "l"(pk(c)));
     return upk(d);
 }
-__device__ __forceinline__ float2 mul2(float2 a, float2 b)
-{
-    unsigned long long d;
-    asm("mul.rn.f32x2 %0, %1, %2;" : "=l"(d) : "l"(pk(a)), "l"(pk(b)));
-    return upk(d);
-}
-__device__ __forceinline__ float2 sub2(float2 a, float2 b)
-{
-    unsigned long long d;
-    asm("sub.rn.f32x2 %0, %1, %2;" : "=l"(d) : "l"(pk(a)), "l"(pk(b)));
-    return upk(d);
-}
 __device__ __forceinline__ float2 add2(float2 a, float2 b)
 {
     unsigned long long d;
@@ -63,139 +52,112 @@ __device__ __forceinline__ float2 add2(float2 a, float2 b)
     return upk(d);
 }
 
-// (1 - exp(-x)) / x for x >= 0, given E = exp(-x): the Taylor series of the
-// left side below x = 1/16 (truncation < x^5/720 < 2^-29 relative), the
-// quotient above (cancellation in 1 - E costs at most 16 ulp there). Both are
-// evaluated and one selected, so that a warp does not diverge.
-__device__ __forceinline__ float one_minus_exp_over_x(float x, float E)
+// (1 - exp(-x)) / x = 1 + x P(x) on [0, 1], P of degree 5 by interpolation at the
+// Chebyshev nodes (within 4e-8 of it in exact arithmetic, 1e-7 in float32). With
+// T e^-x = T - w x it replaces the exponential of a step's optical depth: two ex2
+// and a division less per step, and without their error, which the transmittance
+// multiplied up, the table is within 1e-7 (relative norm) of 64 bits instead of
+// 6 to 8e-7.
+__device__ __forceinline__ float one_minus_exp_over_x(float x)
 {
-    const float series = fmaf(x, fmaf(x, fmaf(x, fmaf(x, 1.0f / 120.0f, -1.0f / 24.0f), 1.0f / 6.0f), -0.5f), 1.0f);
-    const float quot = __fdividef(1.0f - E, x);
-    return x < 0.0625f ? series : quot;
+    float h = 0.00013742418377660215f;
+    h = fmaf(h, x, -0.0013248180039227009f);
+    h = fmaf(h, x, 0.00830117054283619f);
+    h = fmaf(h, x, -0.04165925458073616f);
+    h = fmaf(h, x, 0.16666603088378906f);
+    h = fmaf(h, x, -0.5f);
+    return fmaf(h, x, 1.0f);
 }
 
-// CTAs of 256 threads per SM the register budget of the 8-blob kernel is cut
-// for, and the unroll of the step loop (measured with the packed blob loop:
-// 2 CTAs and 2 steps were fastest).
-#ifndef LF_PRE_MIN_BLOCKS
-#define LF_PRE_MIN_BLOCKS 2
-#endif
-
-// 1: the blob loop in packed FP32 pairs (fma/mul/sub/add .f32x2); 0: scalar.
-#ifndef LF_PRE_PACKED
-#define LF_PRE_PACKED 1
-#endif
-#ifndef LF_PRE_STEP_UNROLL
-#define LF_PRE_STEP_UNROLL 2
-#endif
-constexpr int kPreStepUnroll = LF_PRE_STEP_UNROLL;
+// CTAs of 256 threads per SM the register budget is cut for (the direct render of 9
+// blobs or more: 2), and the unroll of the step loop. Precompute of 16,384 x 512 texels,
+// 8 blobs, 4 samples of 64 steps: 3.73 ms at 2 and 2, 3.75 to 3.82 at 3 or 4 CTAs
+// or unrolled by 1 or 4. Direct render of 8 views of 512^2: 134 us at 3 and 4, 136
+// to 140 elsewhere. Scalar instead of packed FP32 costs the precompute 10% and
+// more.
+constexpr int kPreBlocks = 2, kPreUnroll = 2, kVolBlocks = 3, kVolUnroll = 4;
 
 // Radiance collected along o + t d, t in [0, t_end], by the midpoint rule with
 // p.steps steps of constant density and emission (see the top of the file):
 // (RGB including the background seen through the final transmittance T, and
-// 1 - T).
-template <int BMAX>
+// 1 - T). BP: pairs of blobs.
+template <int BP, int UNROLL>
 __device__ __forceinline__ float4 march(const PrecomputeParams &p, float ox, float oy, float oz, float dx,
                                         float dy, float dz, float t_end)
 {
     const float dt = t_end / (float)p.steps;
-    // per-blob constants of this ray
-    float y0[BMAX], dy0[BMAX], la[BMAX], G[BMAX];
+    // per-blob constants of this ray, in pairs: y0, dy and -(la + log2 dt): the step
+    // length is folded into the densities, g' = g dt = 2^(la + log2 dt - y^2), so the
+    // step's optical depth is sum g' and its weight T (1 - e^-x) / x
+    float2 Y0[BP], DY[BP], NL[BP], G2[BP];
+    const float l2dt = __log2f(dt);
 #pragma unroll
-    for (int k = 0; k < BMAX; ++k) {
-        const float4 bp = p.blob_pos[k];
-        const float a = p.blob_col[k].w;
-        const float fx = ox - bp.x, fy = oy - bp.y, fz = oz - bp.z;
-        const float along = fmaf(fx, dx, fmaf(fy, dy, fz * dz));
-        const float cx = fy * dz - fz * dy, cy = fz * dx - fx * dz, cz = fx * dy - fy * dx;
-        const float perp = fmaf(cx, cx, fmaf(cy, cy, cz * cz));
-        y0[k] = a * fmaf(0.5f, dt, along);
-        dy0[k] = a * dt;
-        la[k] = (k < (int)p.nb) ? fmaf(-a * a, perp, bp.w) : -INFINITY;
-        G[k] = 0.0f;
+    for (int q = 0; q < BP; ++q) {
+        float y0[2], dy0[2], nl[2];
+#pragma unroll
+        for (int h = 0; h < 2; ++h) {
+            const int k = 2 * q + h;
+            const float4 bp = p.blob_pos[k];
+            const float a = p.blob_col[k].w;
+            const float fx = ox - bp.x, fy = oy - bp.y, fz = oz - bp.z;
+            const float along = fmaf(fx, dx, fmaf(fy, dy, fz * dz));
+            const float cx = fy * dz - fz * dy, cy = fz * dx - fx * dz, cz = fx * dy - fy * dx;
+            const float perp = fmaf(cx, cx, fmaf(cy, cy, cz * cz));
+            y0[h] = a * fmaf(0.5f, dt, along);
+            dy0[h] = a * dt;
+            nl[h] = k < (int)p.nb ? -(fmaf(-a * a, perp, bp.w) + l2dt) : INFINITY;
+        }
+        Y0[q] = make_float2(y0[0], y0[1]);
+        DY[q] = make_float2(dy0[0], dy0[1]);
+        NL[q] = make_float2(nl[0], nl[1]);
+        G2[q] = make_float2(0.0f, 0.0f);
     }
 
     float T = 1.0f;
     if (dt > 0.0f) {
-        // dt folded into the densities: g' = g dt = 2^(la + log2 dt - y^2), so the
-        // step's optical depth is sum g' and its weight T (1 - e^-x) / x
-        const float l2dt = __log2f(dt);
-#pragma unroll
-        for (int k = 0; k < BMAX; ++k) la[k] += l2dt;
-#if LF_PRE_PACKED
-        // blobs in pairs: y, y^2, the exponent, the density sum and the
-        // per-blob weights in packed FP32 pairs
-        constexpr int BP = BMAX / 2;
-        float2 Y0[BP], DY[BP], LA[BP], G2[BP];
-#pragma unroll
-        for (int q = 0; q < BP; ++q) {
-            Y0[q] = make_float2(y0[2 * q], y0[2 * q + 1]);
-            DY[q] = make_float2(dy0[2 * q], dy0[2 * q + 1]);
-            LA[q] = make_float2(la[2 * q], la[2 * q + 1]);
-            G2[q] = make_float2(0.0f, 0.0f);
-        }
         float kf = 0.0f;
-#pragma unroll kPreStepUnroll
+#pragma unroll UNROLL
         for (uint32_t st = 0; st < p.steps; ++st, kf += 1.0f) {
             const float2 kf2 = make_float2(kf, kf);
-            float2 g2[BP], sig2 = make_float2(0.0f, 0.0f);
+            float2 g2[BP], sig2;
 #pragma unroll
             for (int q = 0; q < BP; ++q) {
                 const float2 y = fma2(kf2, DY[q], Y0[q]);
-                const float2 arg = sub2(LA[q], mul2(y, y));
-                g2[q] = make_float2(ex2_approx(arg.x), ex2_approx(arg.y));
-                sig2 = add2(sig2, g2[q]);
+                const float2 n = fma2(y, y, NL[q]);
+                g2[q] = make_float2(ex2_approx(-n.x), ex2_approx(-n.y));
+                sig2 = q ? add2(sig2, g2[q]) : g2[0];
             }
-            // step of constant density: x = sigma dt, weight T (1 - e^-x) / x per g'
-            const float xs = sig2.x + sig2.y;
-            const float E = ex2_approx(-xs * kLog2e);
-            const float w = T * one_minus_exp_over_x(xs, E);
+            // step of constant density: x = sigma dt, weight w = T (1 - e^-x) / x per g',
+            // and T e^-x = T - w x
+            const float x = sig2.x + sig2.y;
+            float w = T * one_minus_exp_over_x(x), Tn = fmaf(-w, x, T);
+            if (x > 1.0f) {                              // a dense step, past the polynomial
+                const float E = ex2_approx(-x * kLog2e);
+                w = T * ((1.0f - E) * rcp_approx(x));
+                Tn = T * E;
+            }
+            T = Tn;
             const float2 w2 = make_float2(w, w);
 #pragma unroll
             for (int q = 0; q < BP; ++q) G2[q] = fma2(w2, g2[q], G2[q]);
-            T *= E;
         }
-#pragma unroll
-        for (int q = 0; q < BP; ++q) {
-            G[2 * q] = G2[q].x;
-            G[2 * q + 1] = G2[q].y;
-        }
-#else
-        float kf = 0.0f;
-#pragma unroll kPreStepUnroll
-        for (uint32_t st = 0; st < p.steps; ++st, kf += 1.0f) {
-            float g[BMAX], sig = 0.0f;
-#pragma unroll
-            for (int k = 0; k < BMAX; ++k) {
-                const float y = fmaf(kf, dy0[k], y0[k]);
-                g[k] = ex2_approx(fmaf(-y, y, la[k]));
-                sig += g[k];
-            }
-            // step of constant density: x = sigma dt, weight T (1 - e^-x) / x per g'
-            const float xs = sig;
-            const float E = ex2_approx(-xs * kLog2e);
-            const float w = T * one_minus_exp_over_x(xs, E);
-#pragma unroll
-            for (int k = 0; k < BMAX; ++k) G[k] = fmaf(w, g[k], G[k]);
-            T *= E;
-        }
-#endif
     }
     float L0 = 0.0f, L1 = 0.0f, L2 = 0.0f;
 #pragma unroll
-    for (int k = 0; k < BMAX; ++k) {
+    for (int k = 0; k < 2 * BP; ++k) {
         const float4 bc = p.blob_col[k];
-        L0 = fmaf(G[k], bc.x, L0);
-        L1 = fmaf(G[k], bc.y, L1);
-        L2 = fmaf(G[k], bc.z, L2);
+        const float G = k & 1 ? G2[k >> 1].y : G2[k >> 1].x;
+        L0 = fmaf(G, bc.x, L0);
+        L1 = fmaf(G, bc.y, L1);
+        L2 = fmaf(G, bc.z, L2);
     }
     const float bgw = 0.5f * (1.0f + dz);
     return make_float4(fmaf(T, fmaf(p.bg1[0], bgw, p.bg0[0]), L0), fmaf(T, fmaf(p.bg1[1], bgw, p.bg0[1]), L1),
                        fmaf(T, fmaf(p.bg1[2], bgw, p.bg0[2]), L2), 1.0f - T);
 }
 
-template <int BMAX>
-__global__ void __launch_bounds__(256, BMAX <= 8 ? LF_PRE_MIN_BLOCKS : 1)
+template <int BP>
+__global__ void __launch_bounds__(256, kPreBlocks)
     precompute_kernel(const __grid_constant__ PrecomputeParams p)
 {
     const uint64_t total = (uint64_t)p.rows * p.N;
@@ -252,7 +214,7 @@ __global__ void __launch_bounds__(256, BMAX <= 8 ? LF_PRE_MIN_BLOCKS : 1)
             const float disc = fmaf(b, b, -c);
             const float t_end = disc > 0.0f ? fmaxf(0.0f, sqrtf(disc) - b) : 0.0f;
 
-            const float4 r = march<BMAX>(p, ox, oy, oz, dx, dy, dz, t_end);
+            const float4 r = march<BP, kPreUnroll>(p, ox, oy, oz, dx, dy, dz, t_end);
             acc0 += r.x;
             acc1 += r.y;
             acc2 += r.z;
@@ -270,71 +232,147 @@ __global__ void __launch_bounds__(256, BMAX <= 8 ? LF_PRE_MIN_BLOCKS : 1)
     }
 }
 
-// Direct render of the same volume, one thread per pixel of one view: the
-// pixel's camera ray and its front hit h_o on S (the FP32 steps of the
-// light-field render), the far end of the ray inside S from h_o in FP64 (the
-// FP32 form of |h_o - O|^2 - R^2 cancels for grazing rays), then the
+// Direct render of the same volume, one thread per pixel, in tiles of 16 x 16
+// pixels and warps of 8 x 4 (the rays of a warp run side by side): the pixel's
+// camera ray and its front hit h_o on S (the FP32 steps of the light-field
+// render), the length of the ray inside S from h_o (chord_length), then the
 // integral of the precompute along that ray (one sample, no jitter). Misses
-// store 0.
-template <int BMAX>
-__global__ void __launch_bounds__(256, BMAX <= 8 ? LF_PRE_MIN_BLOCKS : 1)
-    volume_direct_kernel(const __grid_constant__ PrecomputeParams p, const __grid_constant__ ViewK v,
-                         const __grid_constant__ SphereK S, double R)
+// store 0. What bounds it, and the precompute: the FP32 pipe (73% of its cycles
+// with packed pairs at two cycles each, XU 58%, issue 73%).
+constexpr uint32_t kVolTileLog = 4;
+
+// Far end of the segment inside S from the front hit h along unit d: with f = h -
+// O, b = f . d and c = |f|^2 - R^2, -b + sqrt(b^2 - c). In FP32, c cancels for a
+// hit on S and b for a grazing ray; here f . d is summed in double-float and c is
+// error-free (the expansion of unit_hit_df), each then rounded once, so the
+// length is as exact as FP32 holds it. The same in FP64 (some forty operations and
+// a square root at a seventieth of FP32's rate), one launch per view and rows of
+// 256 pixels took 241 us for 8 views of 512^2, 62% hit; this takes 134.
+__device__ __forceinline__ float chord_length(const SphereK &S, float3 h, float3 d)
 {
-    const uint64_t total = (uint64_t)v.width * v.height;
-    const uint64_t stride = (uint64_t)gridDim.x * blockDim.x;
-    for (uint64_t t = (uint64_t)blockIdx.x * blockDim.x + threadIdx.x; t < total; t += stride) {
-        const uint32_t y = (uint32_t)(t / v.width), x = (uint32_t)(t - (uint64_t)y * v.width);
+    const float hv[3] = {h.x, h.y, h.z}, dv[3] = {d.x, d.y, d.z};
+    df f[3], b{0.0f, 0.0f};
+    float small = 0.0f;
+    df sq{0.0f, 0.0f};
+#pragma unroll
+    for (int k = 0; k < 3; ++k) {
+        const df s = two_sum(hv[k], -S.o_hi[k]);
+        f[k] = fast_two_sum(s.h, __fsub_rn(s.l, S.o_lo[k]));
+        b = df_add(b, df_mul(f[k], df{dv[k], 0.0f}));
+        const float p = __fmul_rn(f[k].h, f[k].h);
+        small = __fadd_rn(small, __fmaf_rn(2.0f * f[k].h, f[k].l, __fmaf_rn(f[k].h, f[k].h, -p)));
+        const df t = two_sum(sq.h, p);
+        sq.h = t.h;
+        sq.l = __fadd_rn(sq.l, t.l);
+    }
+    const df r = two_sum(sq.h, -S.r2_h);
+    const float c = __fadd_rn(__fadd_rn(r.h, __fadd_rn(r.l, sq.l)), __fsub_rn(small, S.r2_l));
+    const float disc = __fmaf_rn(b.h, b.h, __fmaf_rn(2.0f * b.h, b.l, -c));
+    return disc > 0.0f ? fmaxf(0.0f, __fsub_rn(__fsqrt_rn(disc), b.h)) : 0.0f;
+}
+
+template <int MAXV>
+struct VolumeParams : PrecomputeParams {
+    SphereK sphere;
+    uint32_t n_views;
+    uint32_t tile_prefix[MAXV + 1];
+    ViewK views[MAXV];
+};
+
+template <int BP, int MAXV>
+__global__ void __launch_bounds__(256, BP <= 4 ? kVolBlocks : 2)
+    volume_direct_kernel(const __grid_constant__ VolumeParams<MAXV> p)
+{
+    uint32_t lo = 0, hi = p.n_views;                     // largest view with tile_prefix <= blockIdx.x
+    while (hi - lo > 1) {
+        const uint32_t mid = (lo + hi) >> 1;
+        if (p.tile_prefix[mid] <= blockIdx.x) lo = mid; else hi = mid;
+    }
+    const ViewK &v = p.views[lo];
+    const uint32_t lt = blockIdx.x - p.tile_prefix[lo];
+    const uint32_t ty = (uint32_t)(((uint64_t)lt * v.div_m) >> v.div_s), tx = lt - ty * v.tiles_x;
+    const uint32_t warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    const uint32_t x = (tx << kVolTileLog) + ((warp & 1u) << 3) + (lane & 7u);
+    const uint32_t y = (ty << kVolTileLog) + ((warp >> 1) << 2) + (lane >> 3);
+    if (x >= v.width || y >= v.height) return;
+    float4 r = make_float4(0.0f, 0.0f, 0.0f, 0.0f);
+    if (!certain_miss(v, x, y)) {
         const float3 d = camera_dir(v, x, y);
         float3 ho, hd;
-        float4 r = make_float4(0.0f, 0.0f, 0.0f, 0.0f);
-        if (intersect_sphere(S, v.eye, d, ho, hd)) {
-            const double f0 = __dsub_rn((double)ho.x, S.o64[0]);
-            const double f1 = __dsub_rn((double)ho.y, S.o64[1]);
-            const double f2 = __dsub_rn((double)ho.z, S.o64[2]);
-            const double b = __dadd_rn(__dadd_rn(__dmul_rn(f0, (double)d.x), __dmul_rn(f1, (double)d.y)),
-                                       __dmul_rn(f2, (double)d.z));
-            const double c = __dsub_rn(__dadd_rn(__dadd_rn(__dmul_rn(f0, f0), __dmul_rn(f1, f1)), __dmul_rn(f2, f2)),
-                                       __dmul_rn(R, R));
-            const double disc = __dsub_rn(__dmul_rn(b, b), c);
-            const double te = disc > 0.0 ? __dadd_rn(-b, __dsqrt_rn(disc)) : 0.0;
-            r = march<BMAX>(p, ho.x, ho.y, ho.z, d.x, d.y, d.z, te > 0.0 ? (float)te : 0.0f);
-        }
-        const uint64_t pix = v.out_offset + t;
-        if (p.C == 4) {
-            reinterpret_cast<float4 *>(p.out)[pix] = r;
-        } else {
-            float *o = p.out + 3 * pix;
-            o[0] = r.x;
-            o[1] = r.y;
-            o[2] = r.z;
-        }
+        if (intersect_sphere(p.sphere, v.eye, d, ho, hd))
+            r = march<BP, kVolUnroll>(p, ho.x, ho.y, ho.z, d.x, d.y, d.z, chord_length(p.sphere, ho, d));
+    }
+    const uint64_t pix = v.out_offset + (uint64_t)y * v.width + x;
+    if (p.C == 4) {
+        reinterpret_cast<float4 *>(p.out)[pix] = r;
+    } else {
+        float *o = p.out + 3 * pix;
+        o[0] = r.x;
+        o[1] = r.y;
+        o[2] = r.z;
     }
 }
 
-cudaError_t launch_volume_direct(const PrecomputeParams &p, const ViewK &v, const SphereK &S, double R,
-                                 cudaStream_t st)
+// One kernel per number of blob pairs: a scene of 3 blobs pays for 4, not 8, one
+// of 9 for 10, not 16.
+template <int MAXV>
+static cudaError_t launch_volume(const VolumeParams<MAXV> &p, unsigned grid, cudaStream_t st)
 {
-    const uint64_t total = (uint64_t)v.width * v.height;
-    const uint64_t blocks = (total + 255) / 256;
-    const unsigned grid = (unsigned)(blocks < (1ull << 20) ? blocks : (1ull << 20));
-    if (p.nb <= 8)
-        volume_direct_kernel<8><<<grid, 256, 0, st>>>(p, v, S, R);
-    else
-        volume_direct_kernel<kMaxBlobs><<<grid, 256, 0, st>>>(p, v, S, R);
-    return cudaGetLastError();
+    static const void *const f[] = {
+        (const void *)volume_direct_kernel<1, MAXV>, (const void *)volume_direct_kernel<2, MAXV>,
+        (const void *)volume_direct_kernel<3, MAXV>, (const void *)volume_direct_kernel<4, MAXV>,
+        (const void *)volume_direct_kernel<5, MAXV>, (const void *)volume_direct_kernel<6, MAXV>,
+        (const void *)volume_direct_kernel<7, MAXV>, (const void *)volume_direct_kernel<8, MAXV>};
+    static_assert(kMaxBlobs == 16, "pairs");
+    void *args[] = {const_cast<VolumeParams<MAXV> *>(&p)};
+    return cudaLaunchKernel(f[p.nb ? (p.nb - 1) / 2 : 0], dim3(grid), dim3(256), args, 0, st);
+}
+
+template <int MAXV>
+static cudaError_t launch_views(const PrecomputeParams &base, const SphereK &S, const lf_view *views, uint32_t n,
+                                double R, const double O[3], cudaStream_t st)
+{
+    static thread_local VolumeParams<MAXV> p;
+    static_cast<PrecomputeParams &>(p) = base;
+    p.sphere = S;
+    lf_launch tile = {1u << kVolTileLog, 1u << kVolTileLog, 8, 0, 0, 0};
+    for (uint32_t v0 = 0; v0 < n;) {
+        // as many views as the parameters hold and a grid of fewer than 2^31 tiles
+        uint64_t tiles = 0;
+        uint32_t nv = 0;
+        for (; nv < (uint32_t)MAXV && v0 + nv < n; ++nv) {
+            p.views[nv] = view_params(views[v0 + nv], tile, R, O);
+            const uint64_t t = (uint64_t)p.views[nv].tiles_x * p.views[nv].tiles_y;
+            if (nv && tiles + t >= (1ull << 31)) break;
+            p.tile_prefix[nv] = (uint32_t)tiles;
+            tiles += t;
+        }
+        p.n_views = nv;
+        const cudaError_t e = launch_volume<MAXV>(p, (unsigned)tiles, st);
+        if (e != cudaSuccess) return e;
+        v0 += nv;
+    }
+    return cudaSuccess;
+}
+
+cudaError_t launch_volume_direct(const PrecomputeParams &p, const lf_view *views, uint32_t n, const SphereK &S, double R,
+                                 const double O[3], cudaStream_t st)
+{
+    return n <= (uint32_t)kSmallViews ? launch_views<kSmallViews>(p, S, views, n, R, O, st)
+                                      : launch_views<kVolumeViews>(p, S, views, n, R, O, st);
 }
 
 cudaError_t launch_precompute(const PrecomputeParams &p, cudaStream_t st)
 {
+    static const void *const f[] = {(const void *)precompute_kernel<1>, (const void *)precompute_kernel<2>,
+                                    (const void *)precompute_kernel<3>, (const void *)precompute_kernel<4>,
+                                    (const void *)precompute_kernel<5>, (const void *)precompute_kernel<6>,
+                                    (const void *)precompute_kernel<7>, (const void *)precompute_kernel<8>};
     const uint64_t total = (uint64_t)p.rows * p.N;
     const uint64_t blocks = (total + 255) / 256;
     const unsigned grid = (unsigned)(blocks < (1ull << 20) ? blocks : (1ull << 20));
-    if (p.nb <= 8)
-        precompute_kernel<8><<<grid, 256, 0, st>>>(p);
-    else
-        precompute_kernel<kMaxBlobs><<<grid, 256, 0, st>>>(p);
-    return cudaGetLastError();
+    void *args[] = {const_cast<PrecomputeParams *>(&p)};
+    return cudaLaunchKernel(f[p.nb ? (p.nb - 1) / 2 : 0], dim3(grid), dim3(256), args, 0, st);
 }
 
 }  // namespace lfk
