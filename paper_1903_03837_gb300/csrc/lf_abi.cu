@@ -204,6 +204,8 @@ PointSetK point_set_of(const float4 *hi, const float4 *lo, const float4 *xy, uin
     P.xy = xy;
     P.n = n;
     P.nf = (float)n;
+    P.nhalf = (float)(0.5 * n);
+    P.zpole = n > 128 ? (float)(1.0 - 17.0 / (double)n) : -1.0f;   // continuous index 8: z = 1 - 17/n
     P.inv_sigma = (float)(1.0 / std::sqrt(sigma2));
     P.sigma2 = (float)(sigma2 * (1.0 - std::ldexp(1.0, -20)));   // a listed point's tent weight is above 0
     P.zone0 = (float)(std::log(std::sqrt(5.0) * 3.14159265358979323846 * n) / (2.0 * std::log(1.6180339887498948482)));
@@ -268,8 +270,9 @@ lf_status run_chunk(const lf_table *t, const lfk::RenderParamsBase &base, const 
     p.total_tiles = (uint32_t)tiles;
     p.total_pixels = 0;
     for (uint32_t v = 0; v < nv; ++v) p.total_pixels += (uint64_t)views[v].width * views[v].height;
-    const unsigned block = L.tile_w * L.tile_h, grid = (unsigned)tiles;
-    if (grid == 0) return LF_OK;
+    if (tiles == 0) return LF_OK;
+    const unsigned block = L.tile_w * L.tile_h;
+    const dim3 grid = lfk::tile_grid(p);
     const cudaError_t e = bwd ? lfk::launch_backward(p, grid, block, st)
                               : lfk::launch_render(t->texel_kind, p, grid, block, st);
     if (e != cudaSuccess) return cuda_fail(e, bwd ? "backward launch" : "render launch");

@@ -21,9 +21,9 @@
 #include "lf_ray.cuh"
 
 // Resident CTAs of kMaxBlock threads per SM the register budget is cut for: the
-// fit's forward and backward take 672 us at 4, 707 at 3, 665 at 5 (which spills).
+// fit's forward and backward take 631 us at 5, 640 at 4, 35 more at 3.
 #ifndef LF_MIN_BLOCKS_BWD
-#define LF_MIN_BLOCKS_BWD 4
+#define LF_MIN_BLOCKS_BWD 5
 #endif
 
 namespace lfk {
@@ -338,7 +338,7 @@ __global__ void __launch_bounds__(kMaxBlock, K == 5 && SEARCH != 9 ? LF_MIN_BLOC
 {
     __shared__ WarpScratch<K> ws[kMaxBlock / 32];
     uint32_t v, tx, ty, px, py;
-    tile_of(p, p.views, p.tile_prefix, p.n_views, blockIdx.x, v, tx, ty);
+    if (!cta_tile(p, v, tx, ty)) return;
     const ViewK &vw = p.views[v];
     if (SEARCH >= 0 && tile_misses(p, vw, tx, ty)) return;   // given indices are checked against every ray
     pixel_of(p, tx, ty, px, py);
@@ -355,20 +355,20 @@ static const void *backward_fn(const RenderParamsBase &p)
 }
 
 template <int MAXV>
-static cudaError_t launch(const RenderParams<MAXV> &p, unsigned grid, unsigned block, cudaStream_t st)
+static cudaError_t launch(const RenderParams<MAXV> &p, dim3 grid, unsigned block, cudaStream_t st)
 {
     void *args[] = {const_cast<RenderParams<MAXV> *>(&p)};
-    cudaError_t e = cudaLaunchKernel(backward_fn<MAXV>(p), dim3(grid), dim3(block), args, 0, st);
+    cudaError_t e = cudaLaunchKernel(backward_fn<MAXV>(p), grid, dim3(block), args, 0, st);
     // nearest sampling may leave near-ties to the exact pass, an upper-hemisphere table rays at the rim of its rows
     if (e == cudaSuccess && !p.nine && !p.idx_in && (p.nearest_only || p.rows_stored)) e = launch_fixup(kF32C4, true, p, st);
     return e;
 }
 
-cudaError_t launch_backward(const RenderParams<kSmallViews> &p, unsigned grid, unsigned block, cudaStream_t st)
+cudaError_t launch_backward(const RenderParams<kSmallViews> &p, dim3 grid, unsigned block, cudaStream_t st)
 {
     return launch(p, grid, block, st);
 }
-cudaError_t launch_backward(const RenderParams<kLargeViews> &p, unsigned grid, unsigned block, cudaStream_t st)
+cudaError_t launch_backward(const RenderParams<kLargeViews> &p, dim3 grid, unsigned block, cudaStream_t st)
 {
     return launch(p, grid, block, st);
 }

@@ -68,6 +68,13 @@ __device__ __forceinline__ float lg2_approx(float x)
     asm("lg2.approx.ftz.f32 %0, %1;" : "=f"(r) : "f"(x));
     return r;
 }
+// 1/x within 1 ulp.
+__device__ __forceinline__ float rcp_approx(float x)
+{
+    float r;
+    asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(r) : "f"(x));
+    return r;
+}
 __device__ __forceinline__ float sqrt_approx(float x)
 {
     float r;
@@ -88,7 +95,7 @@ __device__ __forceinline__ float azimuth_turns(float y, float x)
                                  0.021862957626581192f, -0.004054567310959101f};
     float ax = fabsf(x), ay = fabsf(y);
     float mx = fmaxf(ax, ay), mn = fminf(ax, ay);
-    float a = __fdividef(mn, fmaxf(mx, 1e-30f));
+    float a = mn * rcp_approx(fmaxf(mx, 1e-30f));
     float a2 = a * a;
     float p = kAtanC[7];
 #pragma unroll
@@ -453,7 +460,7 @@ __device__ __forceinline__ Corner lattice_corner(const PointSetK &P, float3 qh)
     float z = qh.z;
     float omz2 = __fmul_rn(__fsub_rn(1.0f, z), __fadd_rn(1.0f, z));
     float t = azimuth_turns(qh.y, qh.x);                            // turns
-    float ic = (P.nf * (1.0f - z) - 1.0f) * 0.5f;                  // continuous index
+    float ic = __fmaf_rn(-P.nhalf, z, P.nhalf - 0.5f);             // continuous index (n(1-z)-1)/2
     int k = __float2int_rd(__fmaf_rn(lg2_approx(omz2), kInvLog2Phi2, P.zone0));
     k = max(2, min(k, kFibN - 3));
     const float4 ab = *reinterpret_cast<const float4 *>(&kZones.z[k].au);
@@ -465,8 +472,10 @@ __device__ __forceinline__ Corner lattice_corner(const PointSetK &P, float3 qh)
     bool pu = u >= ru, pv = v >= rv;
     Corner c;
     c.b = (int32_t)ru * F0 + (int32_t)rv * F1;
-    c.G0 = pu ? (pv ? F0 : -F1) : (pv ? F1 : -F0);
-    c.G1 = pu ? (pv ? F1 : F0) : (pv ? -F0 : -F1);
+    // (F0, F1), (-F1, F0), (F1, -F0), (-F0, -F1) for (pu, pv) = ++, +-, -+, --
+    const int32_t A = pu == pv ? F0 : F1, B = pu == pv ? F1 : F0;
+    c.G0 = pv ? A : -A;
+    c.G1 = pu ? B : -B;
     c.reach = F0 + F1;
     return c;
 }
@@ -1028,16 +1037,6 @@ __device__ __forceinline__ TopK<9> knn9(const PointSetK &P, const SphereK &S, fl
             r.i[m] = 0;
         }
     }
-    return r;
-}
-
-// 1/x by the hardware approximation (within 1 ulp; x here is a sum of tent
-// weights, in (0, 9]): the weights carry a tolerance, not the bits of an IEEE
-// division.
-__device__ __forceinline__ float rcp_approx(float x)
-{
-    float r;
-    asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(r) : "f"(x));
     return r;
 }
 

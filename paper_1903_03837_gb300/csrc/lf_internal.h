@@ -74,7 +74,8 @@ struct PointSetK {
     const float4 *lo;
     const float4 *xy;
     uint32_t n;
-    float nf;
+    float nf, nhalf;         // n and n/2
+    float zpole;             // |z| beyond which points_within scans (8 indices off a pole, or always)
     float inv_sigma;
     float sigma2;
     float zone0;             // log_{Phi^2}(sqrt5*pi*n), the set's part of the zone number

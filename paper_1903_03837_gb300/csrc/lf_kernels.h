@@ -46,6 +46,7 @@ struct RenderParamsBase {
     uint32_t n_views, total_tiles;
     uint32_t tile_w, tile_h, warp_w, order;
     uint32_t tw_log, th_log, ww_log;   // log2 of tile_w, tile_h, warp_w
+    uint32_t grid3;                    // 1: the grid is (tile columns, tile rows, views)
     uint32_t rows_stored;              // origin rows present (upper hemisphere), 0: all
     uint32_t rows_valid;               // rows of the table (M or rows_stored)
     uint32_t nearest_only;             // 1: nearest sampling (K = 1), else 5 or 9 neighbours
@@ -58,12 +59,29 @@ struct RenderParams : RenderParamsBase {
     ViewK views[MAXV];
 };
 
+// The grid of a launch whose views and tiles are set; sets p.grid3. Up to
+// kSmallViews views in raster order take (tile columns, tile rows, views), which
+// spares the kernel the search and the division of a tile number.
+template <int MAXV>
+inline dim3 tile_grid(RenderParams<MAXV> &p)
+{
+    uint32_t tx = 0, ty = 0;
+    for (uint32_t v = 0; v < p.n_views; ++v) {
+        tx = tx > p.views[v].tiles_x ? tx : p.views[v].tiles_x;
+        ty = ty > p.views[v].tiles_y ? ty : p.views[v].tiles_y;
+    }
+    // at most a quarter of the CTAs past a smaller view's tiles
+    p.grid3 = MAXV <= kSmallViews && p.order == 0 && ty < 65536u &&
+              (uint64_t)tx * ty * p.n_views <= (uint64_t)p.total_tiles + p.total_tiles / 3;
+    return p.grid3 ? dim3(tx, ty, p.n_views) : dim3(p.total_tiles);
+}
+
 // lf_render.cu: the forward launch (and, where it may queue rays, the exact pass).
-cudaError_t launch_render(int kind, const RenderParams<kSmallViews> &p, unsigned grid, unsigned block, cudaStream_t st);
-cudaError_t launch_render(int kind, const RenderParams<kLargeViews> &p, unsigned grid, unsigned block, cudaStream_t st);
+cudaError_t launch_render(int kind, const RenderParams<kSmallViews> &p, dim3 grid, unsigned block, cudaStream_t st);
+cudaError_t launch_render(int kind, const RenderParams<kLargeViews> &p, dim3 grid, unsigned block, cudaStream_t st);
 // lf_backward.cu: the gradient scatter.
-cudaError_t launch_backward(const RenderParams<kSmallViews> &p, unsigned grid, unsigned block, cudaStream_t st);
-cudaError_t launch_backward(const RenderParams<kLargeViews> &p, unsigned grid, unsigned block, cudaStream_t st);
+cudaError_t launch_backward(const RenderParams<kSmallViews> &p, dim3 grid, unsigned block, cudaStream_t st);
+cudaError_t launch_backward(const RenderParams<kLargeViews> &p, dim3 grid, unsigned block, cudaStream_t st);
 // lf_fixup.cu: the exact pass over the rays a render or backward launch queued.
 cudaError_t launch_fixup(int kind, bool bwd, const RenderParams<kSmallViews> &p, cudaStream_t st);
 cudaError_t launch_fixup(int kind, bool bwd, const RenderParams<kLargeViews> &p, cudaStream_t st);

@@ -81,8 +81,9 @@ lf_status launch_views(const lfk::RenderParamsBase &base, const lf_launch &L, in
     p.tile_prefix[nv] = (uint32_t)tiles;
     p.n_views = nv;
     p.total_tiles = (uint32_t)tiles;
-    const unsigned block = L.tile_w * L.tile_h, grid = (unsigned)tiles;
-    if (grid == 0) return LF_OK;
+    if (tiles == 0) return LF_OK;
+    const unsigned block = L.tile_w * L.tile_h;
+    const dim3 grid = lfk::tile_grid(p);
     const cudaError_t e = lfk::launch_render(kind, p, grid, block, st);
     if (e != cudaSuccess) return na_fail(LF_ERR_CUDA, "render launch: %s", cudaGetErrorString(e));
     return LF_OK;

@@ -37,6 +37,22 @@ __device__ __forceinline__ void tile_of(const RenderParamsBase &p, const ViewK *
     }
 }
 
+// The CTA's tile: from a grid of (tile columns, tile rows, views) where there is
+// one (grid3: raster order, a few views), else by number. False past a smaller
+// view's tiles.
+template <int MAXV>
+__device__ __forceinline__ bool cta_tile(const RenderParams<MAXV> &p, uint32_t &v, uint32_t &tx, uint32_t &ty)
+{
+    if (MAXV <= kSmallViews && p.grid3) {
+        v = blockIdx.z;
+        tx = blockIdx.x;
+        ty = blockIdx.y;
+        return tx < p.views[v].tiles_x && ty < p.views[v].tiles_y;
+    }
+    tile_of(p, p.views, p.tile_prefix, p.n_views, blockIdx.x, v, tx, ty);
+    return true;
+}
+
 // Pixel of this thread in tile (tx, ty): tile and warp shapes are powers of
 // two, so the mapping is shifts and masks.
 __device__ __forceinline__ void pixel_of(const RenderParamsBase &p, uint32_t tx, uint32_t ty, uint32_t &px,
@@ -64,6 +80,8 @@ __device__ __forceinline__ PointSetK point_set(const RenderParamsBase &p, int s)
     P.xy = s ? p.pd.xy : p.po.xy;
     P.n = s ? p.pd.n : p.po.n;
     P.nf = s ? p.pd.nf : p.po.nf;
+    P.nhalf = s ? p.pd.nhalf : p.po.nhalf;
+    P.zpole = s ? p.pd.zpole : p.po.zpole;
     P.inv_sigma = s ? p.pd.inv_sigma : p.po.inv_sigma;
     P.sigma2 = s ? p.pd.sigma2 : p.po.sigma2;
     P.zone0 = s ? p.pd.zone0 : p.po.zone0;
@@ -127,7 +145,9 @@ __device__ __forceinline__ float z_offset(const PointSetK &P, int32_t c, float q
 __device__ __forceinline__ float dist2_xy(const PointSetK &P, int32_t i, float3 qh, float3 ql, float dz,
                                           uint32_t *status)
 {
-    const float4 a = __ldg(P.xy + LF_DINDEX((uint32_t)(i + kPointPad), P.n + 2 * kPointPad, status, kStatusDebugPoint));
+    // a 32-bit byte offset (below 2^29)
+    const uint32_t e = LF_DINDEX((uint32_t)(i + kPointPad), P.n + 2 * kPointPad, status, kStatusDebugPoint);
+    const float4 a = __ldg(reinterpret_cast<const float4 *>(reinterpret_cast<const char *>(P.xy) + (uint32_t)(e << 4)));
     const float dx = __fadd_rn(__fsub_rn(qh.x, a.x), __fsub_rn(ql.x, a.z));
     const float dy = __fadd_rn(__fsub_rn(qh.y, a.y), __fsub_rn(ql.y, a.w));
     return __fmaf_rn(dx, dx, __fmaf_rn(dy, dy, __fmul_rn(dz, dz)));
@@ -148,13 +168,7 @@ __device__ __forceinline__ int points_within(const PointSetK &P, float3 qh, floa
     const int32_t n = (int32_t)P.n;
     uint2 *w = list;
     const uint2 *const end = list + kListSlots * STRIDE;
-    int32_t scan0 = 0, scan_cnt = n;
-    if (n > 128) {
-        const float icn = (P.nf * (1.0f - qh.z) - 1.0f) * 0.5f, ics = (P.nf * (1.0f + qh.z) - 1.0f) * 0.5f;
-        scan_cnt = icn < 8.0f || ics < 8.0f ? 28 : 0;
-        scan0 = icn < 8.0f ? 0 : n - 28;
-    }
-    if (scan_cnt == 0) {
+    if (!(fabsf(qh.z) > P.zpole)) {
         const Corner c = lattice_corner(P, qh);
         if constexpr (RANK) {
             if (!scan_source(P, qh, src)) src = window_of(P, c);
@@ -193,6 +207,7 @@ __device__ __forceinline__ int points_within(const PointSetK &P, float3 qh, floa
         }
     } else {
         if constexpr (RANK) scan_source(P, qh, src);
+        const int32_t scan_cnt = n > 128 ? 28 : n, scan0 = n > 128 && qh.z < 0.0f ? n - 28 : 0;
 #pragma unroll 4
         for (int j = 0; j < scan_cnt; ++j) {
             const int32_t i = scan0 + j;
@@ -353,8 +368,11 @@ __device__ __forceinline__ bool ray_lists(const RenderParamsBase &p, const ViewK
     __shared__ int s_stash[IDX ? IDX * kMaxBlock : 1];   // the origins' indices during the second search
     float3 ho, hd;
     if (!intersect_sphere(p.sphere, v.eye, d, ho, hd)) return false;
-    // One copy of the search serves both sets (instruction-cache footprint).
-#pragma unroll 1
+    // Without ranking, a copy of the search for each set: their constants are
+    // operands of the instructions (64 uneven views 3.44 -> 3.29 ms); the ranked
+    // searches are too long for the instruction cache twice and share one copy.
+    constexpr int kSetUnroll = IDX == 0 ? 2 : 1;
+#pragma unroll kSetUnroll
     for (int s = 0; s < 2; ++s) {
         const PointSetK P = point_set(p, s);
         uint2 *list = lists + s * kListSlots * STRIDE;

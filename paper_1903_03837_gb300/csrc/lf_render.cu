@@ -13,24 +13,25 @@
 // views (4.10 against 3.46 ms), so a launch is never persistent.
 //
 // What bounds it: instruction issue (75% of the issue slots on a 1080p frame of
-// a 65,536 x 1,024 FP16 table, ALU pipe 48%, FMA 38%, DRAM 3%). An image lists
+// a 65,536 x 1,024 FP16 table, ALU pipe 46%, FMA 38%, DRAM 3%). An image lists
 // the points within the kernel's radius (lf_ray.cuh) instead of ranking the
-// nearest ones and certifying the order: that frame 0.052 ms instead of 0.119
-// (1,450 thread instructions per hit ray instead of 2,680, and no exact pass), a
-// 2 x 3840 x 2160 frame of a 262,144 x 4,096 E4M3 table 0.287 instead of 0.547,
-// 64 uneven views of a 16,384 x 512 FP16 table 3.47 instead of 6.46.
+// nearest ones and certifying the order: that frame 0.051 ms instead of 0.119
+// (1,430 thread instructions per hit ray instead of 2,680, and no exact pass), a
+// 2 x 3840 x 2160 frame of a 262,144 x 4,096 E4M3 table 0.252 instead of 0.547,
+// 64 uneven views of a 16,384 x 512 FP16 table 3.19 instead of 6.46. Per hit ray of
+// that frame: blend 381, candidates' distances 250, lattice corners 267, unit hits
+// 182, camera and hits 107, lists 76.
 #include <cuda_fp16.h>
 #include <cuda_runtime.h>
 
 #include "lf_ray.cuh"
 
-// Resident CTAs of kMaxBlock threads per SM the register budget is cut for: 4
-// (64 registers) is fastest on single frames of every storage form; 3 is 6 to 16%
-// slower there, 5 is 4% faster on the 4K stereo frame and 1 to 3% slower on the
-// small ones, 6 slower everywhere. The variants that rank indices spill 72 bytes
-// at 4 and are as fast at 3.
+// Resident CTAs of kMaxBlock threads per SM the register budget of the unranked
+// kernels is cut for: 5 (48 registers, 8 bytes spilled) against 4 takes the 4K
+// stereo frame from 277 to 252 us and the 64 views from 3.29 to 3.19 ms; 6 is 2%
+// slower than 5. The variants that rank 5 indices spill 80 bytes at 4.
 #ifndef LF_MIN_BLOCKS
-#define LF_MIN_BLOCKS 4
+#define LF_MIN_BLOCKS 5
 #endif
 
 namespace lfk {
@@ -82,6 +83,8 @@ __device__ __forceinline__ float4 blend(const RenderParamsBase &p, const RayList
     float wd[kListSlots], sd = 0.0f;
 #pragma unroll
     for (int b = 0; b < kListSlots; ++b) {
+        wd[b] = 0.0f;
+        if (b == kListSlots - 1 && !five) break;
         const uint2 e = L.e[1][b][threadIdx.x];
         const bool live = b < cd;
         jo[b] = b == 0 ? (live ? e.x * kTexelBytes<DT> : 0u) : (live ? (Off)(e.x * kTexelBytes<DT>) : jo[0]);
@@ -99,15 +102,15 @@ __device__ __forceinline__ float4 blend(const RenderParamsBase &p, const RayList
         so += w;
         float s = w;
         if constexpr (DT == kF16C4 || DT == kE4M3C4) s *= __ldg(p.scales + i);
-        const Off row = (Off)i * (Off)p.N * (Off)kTexelBytes<DT>;
-        float2 in_xy = make_float2(0.f, 0.f), in_zw = make_float2(0.f, 0.f);
+        const Off row = (Off)i * ((Off)p.N * (Off)kTexelBytes<DT>);
+        float2 in_xy, in_zw;
 #pragma unroll
         for (int b = 0; b < kListSlots; ++b) {
             if (b == kListSlots - 1 && !five) break;
             const float4 t = texel_at<DT, Off>(p, row + jo[b]);
             const float2 w2 = make_float2(wd[b], wd[b]);
-            in_xy = ffma2(w2, make_float2(t.x, t.y), in_xy);
-            in_zw = ffma2(w2, make_float2(t.z, t.w), in_zw);
+            in_xy = ffma2(w2, make_float2(t.x, t.y), b ? in_xy : make_float2(0.f, 0.f));
+            in_zw = ffma2(w2, make_float2(t.z, t.w), b ? in_zw : make_float2(0.f, 0.f));
         }
         const float2 s2 = make_float2(s, s);
         acc_xy = ffma2(s2, in_xy, acc_xy);
@@ -147,7 +150,9 @@ __device__ __forceinline__ void render_ray(const RenderParamsBase &p, const View
     }
 }
 
-// Every pixel of a tile outside the view's screen bound of S.
+// A pixel of a tile outside the view's screen bound of S. (One warp storing the
+// whole tile while the others leave takes fewer instructions and more time: 9% on
+// the 4K stereo frame, 59% of whose tiles miss.)
 template <int IDX>
 __device__ __forceinline__ void store_miss(const RenderParamsBase &p, const ViewK &v, uint32_t px, uint32_t py)
 {
@@ -163,12 +168,12 @@ __device__ __forceinline__ void store_miss(const RenderParamsBase &p, const View
 }
 
 template <int DT, int MAXV, int IDX, typename Off>
-__global__ void __launch_bounds__(kMaxBlock, IDX == 9 ? 2 : LF_MIN_BLOCKS)
+__global__ void __launch_bounds__(kMaxBlock, IDX == 9 ? 2 : IDX == 5 ? 4 : LF_MIN_BLOCKS)
     render_kernel(const __grid_constant__ RenderParams<MAXV> p)
 {
     __shared__ RayLists L;
     uint32_t v, tx, ty, px, py;        // v, tx, ty: the same in the whole CTA (uniform registers)
-    tile_of(p, p.views, p.tile_prefix, p.n_views, blockIdx.x, v, tx, ty);
+    if (!cta_tile(p, v, tx, ty)) return;
     const ViewK &vw = p.views[v];
     pixel_of(p, tx, ty, px, py);
     const bool active = px < vw.width && py < vw.height;
@@ -213,19 +218,19 @@ static bool may_defer(const RenderParamsBase &p)
 }
 
 template <int MAXV>
-static cudaError_t launch(int kind, const RenderParams<MAXV> &p, unsigned grid, unsigned block, cudaStream_t st)
+static cudaError_t launch(int kind, const RenderParams<MAXV> &p, dim3 grid, unsigned block, cudaStream_t st)
 {
     void *args[] = {const_cast<RenderParams<MAXV> *>(&p)};
-    cudaError_t e = cudaLaunchKernel(render_fn<MAXV>(kind, p), dim3(grid), dim3(block), args, 0, st);
+    cudaError_t e = cudaLaunchKernel(render_fn<MAXV>(kind, p), grid, dim3(block), args, 0, st);
     if (e == cudaSuccess && may_defer(p)) e = launch_fixup(kind, false, p, st);
     return e;
 }
 
-cudaError_t launch_render(int kind, const RenderParams<kSmallViews> &p, unsigned grid, unsigned block, cudaStream_t st)
+cudaError_t launch_render(int kind, const RenderParams<kSmallViews> &p, dim3 grid, unsigned block, cudaStream_t st)
 {
     return launch(kind, p, grid, block, st);
 }
-cudaError_t launch_render(int kind, const RenderParams<kLargeViews> &p, unsigned grid, unsigned block, cudaStream_t st)
+cudaError_t launch_render(int kind, const RenderParams<kLargeViews> &p, dim3 grid, unsigned block, cudaStream_t st)
 {
     return launch(kind, p, grid, block, st);
 }
