@@ -10,6 +10,7 @@ from __future__ import annotations
 
 import ctypes as C
 import os
+import struct
 import threading
 from typing import Optional, Sequence
 
@@ -71,6 +72,8 @@ _lock = threading.Lock()
 def lib():
     """Load liblumipath.so (building it with nvcc if it is missing or stale)."""
     global _lib
+    if _lib is not None:
+        return _lib
     with _lock:
         if _lib is None:
             path = os.environ.get("LUMIPATH_LIB")      # another build of the library (e.g. debug)
@@ -124,11 +127,24 @@ def _check(status: int):
         raise LfError(status, lib().lf_last_error().decode(errors="replace"))
 
 
+_VIEW = struct.Struct("=14f2IQ")        # lf_view (its fields leave no padding)
+assert _VIEW.size == C.sizeof(lf_view)
+
+
 def make_views(views: Sequence) -> "C.Array":
     """lf_view array from objects with eye/right/up/forward/tan_half_x/
     tan_half_y/width/height/out_offset attributes (e.g. lf_inputs.View)."""
     arr = (lf_view * len(views))()
     for k, v in enumerate(views):
+        try:
+            # one call packs a view; what struct refuses (a float beyond FP32, a size
+            # beyond its field) takes ctypes' own conversions below
+            if len(v.eye) == len(v.right) == len(v.up) == len(v.forward) == 3:
+                _VIEW.pack_into(arr, k * _VIEW.size, *v.eye, *v.right, *v.up, *v.forward, v.tan_half_x, v.tan_half_y,
+                                v.width, v.height, v.out_offset)
+                continue
+        except (struct.error, OverflowError, TypeError):
+            pass
         a = arr[k]
         a.eye[:] = list(v.eye)
         a.right[:] = list(v.right)
@@ -154,26 +170,22 @@ def lf_create_table(desc: lf_table_desc, radiance_ptr: int, scales_ptr: Optional
 
 
 def lf_render(table: int, views, n_views: int, out_ptr: int, idx_ptr: Optional[int], stream: int = 0):
-    _check(lib().lf_render(C.c_void_p(table), views, n_views, C.c_void_p(out_ptr),
-                           C.c_void_p(idx_ptr or None), C.c_void_p(stream or None)))
+    _check((_lib or lib()).lf_render(table, views, n_views, out_ptr, idx_ptr or None, stream or None))
 
 
 def lf_render_f16(table: int, views, n_views: int, out_ptr: int, idx_ptr: Optional[int], stream: int = 0):
-    _check(lib().lf_render_f16(C.c_void_p(table), views, n_views, C.c_void_p(out_ptr),
-                               C.c_void_p(idx_ptr or None), C.c_void_p(stream or None)))
+    _check((_lib or lib()).lf_render_f16(table, views, n_views, out_ptr, idx_ptr or None, stream or None))
 
 
 def lf_render_backward(table: int, views, n_views: int, grad_out_ptr: int, grad_table_ptr: int,
                        stream: int = 0):
-    _check(lib().lf_render_backward(C.c_void_p(table), views, n_views, C.c_void_p(grad_out_ptr),
-                                    C.c_void_p(grad_table_ptr), C.c_void_p(stream or None)))
+    _check((_lib or lib()).lf_render_backward(table, views, n_views, grad_out_ptr, grad_table_ptr, stream or None))
 
 
 def lf_render_backward_idx(table: int, views, n_views: int, grad_out_ptr: int, idx_ptr: int,
                            grad_table_ptr: int, stream: int = 0):
-    _check(lib().lf_render_backward_idx(C.c_void_p(table), views, n_views, C.c_void_p(grad_out_ptr),
-                                        C.c_void_p(idx_ptr), C.c_void_p(grad_table_ptr),
-                                        C.c_void_p(stream or None)))
+    _check((_lib or lib()).lf_render_backward_idx(table, views, n_views, grad_out_ptr, idx_ptr, grad_table_ptr,
+                                                  stream or None))
 
 
 def lf_destroy(table: Optional[int]):

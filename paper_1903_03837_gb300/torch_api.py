@@ -33,6 +33,9 @@ def _need_cuda(t: torch.Tensor, name: str):
 
 
 def total_pixels(views: Sequence) -> int:
+    if len(views) == 1:
+        v = views[0]
+        return int(v.out_offset) + int(v.width) * int(v.height)
     return max(int(v.out_offset) + int(v.width) * int(v.height) for v in views)
 
 
