@@ -17,7 +17,7 @@ from . import build as _build
 CACHE = os.path.join(_build.BUILD, "autotune.json")
 _lock = threading.Lock()
 
-# (tile_w, tile_h, warp_w, order, persistent)
+# (tile_w, tile_h, warp_w, order, persistent; the last has no effect on a launch)
 CANDIDATES = [
     (16, 16, 8, 0, 0), (16, 16, 8, 1, 0), (16, 16, 8, 0, 1), (16, 16, 8, 1, 1),
     (32, 8, 8, 0, 0), (32, 8, 8, 1, 1), (8, 32, 8, 0, 0), (16, 8, 8, 0, 0),

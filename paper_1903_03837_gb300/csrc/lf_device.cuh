@@ -555,17 +555,12 @@ struct TopK {
 };
 using Top5 = TopK<5>;
 
-// The 5 nearest points of the unit hit of h (qh + ql) in (distance, index)
-// order, with their double-float squared distances; cnt = min(5, n). This is
-// the render kernels' fast path: tier 1 and its order certificate, and when
-// that fails a short tier 2 over the tier-1 top 6. When tier 2 cannot settle
-// the order either, `uncertain` is set and the result is meaningless; the
-// render kernel queues the ray for the exact pass (coop_knn5 in a kernel of
-// its own). Neither the exact ranking nor any FP64 code sits in the render
-// kernel: a rarely taken path there costs the common path registers (spills),
-// and run by one lane it holds its warp and CTA for tens of thousands of
-// cycles (FP64 division and square root alone take hundreds of cycles each on
-// this GPU).
+// The 5 nearest points of the unit hit qh + ql in (distance, index) order, with
+// their double-float squared distances; cnt = min(5, n): tier 1 and its order
+// certificate, and when that fails a short tier 2 over the tier-1 top 6. When tier
+// 2 cannot settle the order either, `uncertain` is set and the result is
+// meaningless. The fixup kernel searches the sets that a render kernel settled
+// (rank5) with it.
 __device__ __forceinline__ Top5 knn5(const PointSetK &P, float3 qh, float3 ql, const Source &src, uint32_t *status,
                                      bool &uncertain)
 {

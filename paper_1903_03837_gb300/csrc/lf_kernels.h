@@ -35,12 +35,13 @@ struct RenderParamsBase {
     const float *grad_out;         // backward: [P][C]
     float *grad;                   // backward: [M][N][C]
     uint32_t *status;
-    // Rays whose fast-path order was not certain: the render kernel queues
-    // them here and the fixup kernel that follows it on the stream renders
-    // them (more than defer_cap in one launch: the fixup renders every ray).
+    // Rays whose neighbour order (or, for nearest sampling and upper-hemisphere
+    // tables, neighbour) was not certain: the render kernel queues them here and the
+    // fixup kernel that follows it on the stream finishes them (more than defer_cap
+    // in one launch: the fixup takes every ray).
     unsigned long long *defer_count;   // rays queued in this launch (reset by the fixup kernel)
     uint32_t *defer_done;              // fixup CTAs finished
-    unsigned long long *defer_items;   // [defer_cap]: view << 32 | y << 16 | x
+    unsigned long long *defer_items;   // [defer_cap]: pend << 48 | view << 32 | y << 16 | x
     uint32_t defer_cap;
     uint64_t total_pixels;             // pixels of all views of the launch
     uint32_t n_views, total_tiles;
