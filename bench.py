@@ -441,8 +441,7 @@ def run_ours(args, rank: int, world: int):
                      "frac": achieved / peak, "traffic": recorded_traffic(args.dtype),
                      "peak_source": f"{peak_kind} hbm_gbs",
                      "algorithmic_bytes_per_launch": bytes_per_launch,
-                     "kernel": f"lfk::render_kernel<{args.dtype}> with the lfk::fixup_kernel that follows it "
-                               f"(the exact pass of the rays left uncertain); timed together, per step",
+                     "kernel": f"lfk::render_kernel<{args.dtype}>",
                      "avg_launch_ms": avg_launch_s * 1e3,
                      "compulsory_bytes_per_launch": compulsory["bytes"] if compulsory else None,
                      "l2_bytes_per_launch": recorded_counter(args.dtype, "l2_bytes_per_launch"),
@@ -553,7 +552,7 @@ def run_precompute(args):
                          "peak_source": f"derived: {sms} SMs x 128 FP32 lanes x {mhz:.0f} MHz",
                          "exp2_per_s_T": exp2s / (ms * 1e-3) / 1e12,
                          "exp2_frac_of_32_per_sm_clk": exp2s / (ms * 1e-3) / 1e12 / xu_peak,
-                         "kernel": "lfk::precompute_kernel<8>"},
+                         "kernel": "lfk::precompute_kernel<4 blob pairs>"},
             "light_field_vs_direct": versus}
 
 
