@@ -270,6 +270,31 @@ __device__ __forceinline__ bool rank5(const PointSetK &P, float3 qh, float3 ql, 
     return sure;
 }
 
+// The list of a scanned set from its ranked indices: the points within sigma are
+// among the 5 nearest (even where the order is not certain: the 6th lies beyond
+// 1.04 sigma), listed by index as the scan would.
+template <int STRIDE, int K>
+__device__ __forceinline__ int list_ranked(const PointSetK &P, float3 qh, float3 ql, const int32_t (&ix)[K], uint2 *list)
+{
+    float d2[kListSlots];
+    int c = 0;
+#pragma unroll
+    for (int m = 0; m < kListSlots; ++m) {
+        d2[m] = dist2_df(P, max(ix[m], 0), qh, ql);
+        if (ix[m] < 0) d2[m] = 8.0f;
+    }
+#pragma unroll
+    for (int m = 0; m < kListSlots; ++m) {
+        if (!(d2[m] < P.sigma2) || ix[m] < 0) continue;
+        int at = 0;
+#pragma unroll
+        for (int k = 0; k < kListSlots; ++k) at += d2[k] < P.sigma2 && ix[k] >= 0 && ix[k] < ix[m] ? 1 : 0;
+        list[at * STRIDE] = make_uint2((uint32_t)ix[m], __float_as_uint(d2[m]));
+        ++c;
+    }
+    return c;
+}
+
 // Tent weight of a listed point.
 __device__ __forceinline__ float tent(float d2, float inv_sigma)
 {
@@ -399,7 +424,14 @@ __device__ __forceinline__ bool ray_lists(const RenderParamsBase &p, const ViewK
         unit_hit_df(p.sphere, s ? hd : ho, qh, ql);
         Source src;
         float pre[kWindow];
-        int c = points_within<IDX == 5, STRIDE>(P, qh, ql, list, p.status, src, pre);
+        int c = 0;
+        // a ranking of a whole set (at most 128 points) has scanned it already: 16% of
+        // an index render of 110 directions
+        const bool whole = IDX != 0 && P.n <= 128;
+        if (whole)
+            scan_source(P, qh, src);
+        else
+            c = points_within<IDX == 5, STRIDE>(P, qh, ql, list, p.status, src, pre);
         int32_t ix[IDX ? IDX : 1];
         if constexpr (IDX == 5) {
             if (!rank5(P, qh, ql, src, p.status, pre, ix)) pend |= 1u << s;
@@ -407,6 +439,9 @@ __device__ __forceinline__ bool ray_lists(const RenderParamsBase &p, const ViewK
             const TopK<9> r = knn9(P, p.sphere, s ? hd : ho, qh, ql, candidate_source(P, qh), p.status);
 #pragma unroll
             for (int m = 0; m < 9; ++m) ix[m] = r.i[m];
+        }
+        if constexpr (IDX != 0) {
+            if (whole) c = list_ranked<STRIDE>(P, qh, ql, ix, list);
         }
         if (p.nearest_only) {
             if (!nearest_listed<STRIDE>(P, qh, ql, list, c)) pend |= (1u << s) | kPendImage;
