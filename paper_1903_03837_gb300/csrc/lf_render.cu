@@ -70,7 +70,11 @@ struct RayLists {
 // up to there a lane without a neighbour reads its first direction's column (a
 // texel it loads anyway) with weight 0: a branch around the load costs more than
 // the load. Every texel is finite (the FP32 table is the caller's promise; FP16
-// and E4M3 codes are finite by construction), so such a tap adds exactly 0.
+// and E4M3 codes are finite by construction), so such a tap adds exactly 0. The
+// direction weights are a quarter of the tent: a set's weights sum to at most 1.32,
+// so every sum stays below 0.44 of the largest texel and cannot overflow (an
+// infinite sum times the weight 0 of an origin slot past the list would be NaN). A
+// power of two changes no bit of the quotient and takes no instruction.
 // Every lane of the warp calls it.
 template <int DT, typename Off>
 __device__ __forceinline__ float4 blend(const RenderParamsBase &p, const RayLists &L, int co, int cd)
@@ -88,7 +92,7 @@ __device__ __forceinline__ float4 blend(const RenderParamsBase &p, const RayList
         const uint2 e = L.e[1][b][threadIdx.x];
         const bool live = b < cd;
         jo[b] = b == 0 ? (live ? e.x * kTexelBytes<DT> : 0u) : (live ? (Off)(e.x * kTexelBytes<DT>) : jo[0]);
-        wd[b] = live ? tent(__uint_as_float(e.y), p.pd.inv_sigma) : 0.0f;
+        wd[b] = live ? quarter_tent(__uint_as_float(e.y), p.pd.inv_sigma) : 0.0f;
         sd += wd[b];
     }
     float2 acc_xy = make_float2(0.f, 0.f), acc_zw = make_float2(0.f, 0.f);
