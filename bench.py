@@ -55,7 +55,7 @@ def measured_peaks():
 
 
 RENDER_SOURCES = ("paper_1903_03837_gb300/csrc/lf_render.cu", "paper_1903_03837_gb300/csrc/lf_ray.cuh",
-                  "paper_1903_03837_gb300/csrc/lf_device.cuh",
+                  "paper_1903_03837_gb300/csrc/lf_device.cuh", "paper_1903_03837_gb300/csrc/lf_df.cuh",
                   "paper_1903_03837_gb300/csrc/lf_kernels.h", "paper_1903_03837_gb300/csrc/lf_internal.h",
                   "include/lumipath.h", "paper_1903_03837_gb300/build.py")
 

@@ -197,7 +197,7 @@ ViewK view_params(const lf_view &w, const lf_launch &L, double R, const double O
 
 PointSetK point_set_of(const float4 *hi, const float4 *lo, const float4 *xy, uint32_t n)
 {
-    const double sigma2 = 12.566370614359172953850573533118 / (double)n, step = 2.0 / (double)n;
+    const double sigma2 = 12.566370614359172953850573533118 / (double)n;
     PointSetK P;
     P.hi = hi;
     P.lo = lo;
@@ -209,9 +209,7 @@ PointSetK point_set_of(const float4 *hi, const float4 *lo, const float4 *xy, uin
     P.inv_sigma = (float)(1.0 / std::sqrt(sigma2));
     P.sigma2 = (float)(sigma2 * (1.0 - std::ldexp(1.0, -20)));   // a listed point's tent weight is above 0
     P.zone0 = (float)(std::log(std::sqrt(5.0) * 3.14159265358979323846 * n) / (2.0 * std::log(1.6180339887498948482)));
-    P.zstep_h = (float)step;
-    P.zstep_l = (float)(step - (double)P.zstep_h);
-    P.zhalf = (float)(0.5 * step);
+    fill_z_steps(P);
     return P;
 }
 

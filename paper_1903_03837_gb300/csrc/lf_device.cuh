@@ -11,6 +11,7 @@
 #include <cuda_runtime.h>
 #include <stdint.h>
 
+#include "lf_df.cuh"
 #include "lf_internal.h"
 
 namespace lfk {
@@ -204,34 +205,8 @@ __device__ __forceinline__ int approx_mask(const ViewK &v, uint32_t x, uint32_t 
 }
 
 // ---------------------------------------------------------------------------
-// Double-float arithmetic (value = hi + lo, about 48 significant bits).
+// Unit hits
 // ---------------------------------------------------------------------------
-struct df { float h, l; };
-__device__ __forceinline__ df two_sum(float a, float b)
-{
-    float s = __fadd_rn(a, b);
-    float bb = __fsub_rn(s, a);
-    float e = __fadd_rn(__fsub_rn(a, __fsub_rn(s, bb)), __fsub_rn(b, bb));
-    return {s, e};
-}
-__device__ __forceinline__ df fast_two_sum(float a, float b)
-{
-    float s = __fadd_rn(a, b);
-    return {s, __fsub_rn(b, __fsub_rn(s, a))};
-}
-__device__ __forceinline__ df df_add(df x, df y)
-{
-    df s = two_sum(x.h, y.h);
-    return fast_two_sum(s.h, __fadd_rn(s.l, __fadd_rn(x.l, y.l)));
-}
-__device__ __forceinline__ df df_mul(df x, df y)
-{
-    float p = __fmul_rn(x.h, y.h);
-    float e = __fmaf_rn(x.h, y.h, -p);
-    e = __fmaf_rn(x.h, y.l, __fmaf_rn(x.l, y.h, e));
-    return fast_two_sum(p, e);
-}
-
 // Unit vector (h - O)/|h - O| as hi/lo float3 pairs by a double-float Newton
 // step from rsqrt (|error| about 2^-44); used when h lies far off the sphere.
 __device__ __forceinline__ void unit_hit_df_newton(df f[3], float3 &qh, float3 &ql)

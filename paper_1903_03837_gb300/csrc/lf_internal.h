@@ -4,6 +4,8 @@
 
 #include <stdint.h>
 
+#include <cmath>
+
 #include "lumipath.h"
 
 namespace lfk {
@@ -68,7 +70,7 @@ constexpr int32_t kPointPad = 64;
 // One SF point set: p_i as hi/lo float4 pairs (w unused) and, for the searches
 // that need x and y only (z is linear in i), as one float4 (x_hi, y_hi, x_lo,
 // y_lo) at entry kPointPad + i; n, n as float, the kernel radius sigma = sqrt(4*pi/n) as its
-// reciprocal and square (less 2^-20 of it), and the z step 2/n as a hi/lo pair with its half 1/n.
+// reciprocal and square (less 2^-20 of it), and the z step 2/n and z_0 = 1 - 1/n as hi/lo pairs.
 struct PointSetK {
     const float4 *hi;
     const float4 *lo;
@@ -79,8 +81,25 @@ struct PointSetK {
     float inv_sigma;
     float sigma2;
     float zone0;             // log_{Phi^2}(sqrt5*pi*n), the set's part of the zone number
-    float zstep_h, zstep_l, zhalf;
+    float zstep_h, zstep_l, z0_h, z0_l;
+    float zstep_c, zstep_r;  // the z step as 11 bits and the rest
+    float zgrid;             // 1.5 2^23 units of the last of those bits: adding and taking it off rounds to them
 };
+
+inline void fill_z_steps(PointSetK &P)
+{
+    const double step = 2.0 / (double)P.n;
+    int e;
+    std::frexp(step, &e);
+    const double unit = std::ldexp(1.0, e - 11);
+    P.zstep_h = (float)step;
+    P.zstep_l = (float)(step - (double)P.zstep_h);
+    P.z0_h = (float)(1.0 - 0.5 * step);
+    P.z0_l = (float)(1.0 - 0.5 * step - (double)P.z0_h);
+    P.zstep_c = (float)(std::rint(step / unit) * unit);
+    P.zstep_r = (float)(step - (double)P.zstep_c);
+    P.zgrid = (float)std::ldexp(1.5 * unit, 23);
+}
 
 // Argument checks and view set-up shared by the entry points (lf_abi.cu): a
 // failed check sets the calling thread's lf_last_error() message.

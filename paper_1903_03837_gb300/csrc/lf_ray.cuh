@@ -87,7 +87,11 @@ __device__ __forceinline__ PointSetK point_set(const RenderParamsBase &p, int s)
     P.zone0 = s ? p.pd.zone0 : p.po.zone0;
     P.zstep_h = s ? p.pd.zstep_h : p.po.zstep_h;
     P.zstep_l = s ? p.pd.zstep_l : p.po.zstep_l;
-    P.zhalf = s ? p.pd.zhalf : p.po.zhalf;
+    P.z0_h = s ? p.pd.z0_h : p.po.z0_h;
+    P.z0_l = s ? p.pd.z0_l : p.po.z0_l;
+    P.zstep_c = s ? p.pd.zstep_c : p.po.zstep_c;
+    P.zstep_r = s ? p.pd.zstep_r : p.po.zstep_r;
+    P.zgrid = s ? p.pd.zgrid : p.po.zgrid;
     return P;
 }
 
@@ -128,18 +132,6 @@ __device__ __forceinline__ void defer_push(const RenderParamsBase &p, uint32_t v
 // ---------------------------------------------------------------------------
 constexpr int kListSlots = 5;
 
-// q_z - z_c of the unit hit and SF point c (z_c = 1 - (2 c + 1) / n), to about
-// 2^-24 of itself: c * 2/n as an exact product sum, every cancelling step
-// exact.
-__device__ __forceinline__ float z_offset(const PointSetK &P, int32_t c, float qzh, float qzl)
-{
-    const float cf = __int2float_rn(c);                  // exact: c <= 2^24
-    const float t = __fmul_rn(cf, P.zstep_h);
-    const float e = __fadd_rn(__fmaf_rn(cf, P.zstep_h, -t), __fmaf_rn(cf, P.zstep_l, P.zhalf));
-    const df s = two_sum(t, -1.0f);
-    return __fadd_rn(__fadd_rn(qzh, s.h), __fadd_rn(__fadd_rn(qzl, s.l), e));
-}
-
 // Squared distance of the unit hit to point i (-kPointPad .. n + kPointPad - 1;
 // far outside [0, n)), with dz = q_z - z_i at hand.
 __device__ __forceinline__ float dist2_xy(const PointSetK &P, int32_t i, float3 qh, float3 ql, float dz,
@@ -176,13 +168,12 @@ __device__ __forceinline__ int points_within(const PointSetK &P, float3 qh, floa
         // never taken: keeps every access within the padded cache whatever the hit's values are
         const int32_t reach = RANK ? 2 * c.reach : c.reach;
         if (c.b - reach < -kPointPad || c.b + reach >= n + kPointPad) return 0;
-        const float zb = z_offset(P, c.b, qh.z, ql.z);
-        const float z0 = __fmul_rn(__int2float_rn(c.G0), P.zstep_h);
-        const float z1 = __fmul_rn(__int2float_rn(c.G1), P.zstep_h);
-        const float zp = __fadd_rn(zb, z0), zm = __fsub_rn(zb, z0);
+        const ZOffset zb = z_offset(P, c.b, qh.z, ql.z);
+        const float g0 = __int2float_rn(c.G0), g1 = __int2float_rn(c.G1);      // their sums below are exact
         const int32_t b = c.b, ip = b + c.G0, im = b - c.G0;
         const int32_t idx[7] = {b, b + c.G1, ip, ip + c.G1, b - c.G1, im + c.G1, im};
-        const float dz[7] = {zb, __fadd_rn(zb, z1), zp, __fadd_rn(zp, z1), __fsub_rn(zb, z1), __fadd_rn(zm, z1), zm};
+        const float dz[7] = {__fadd_rn(zb.c, zb.r), z_at(P, zb, g1),  z_at(P, zb, g0), z_at(P, zb, g0 + g1),
+                             z_at(P, zb, -g1),      z_at(P, zb, g1 - g0), z_at(P, zb, -g0)};
         float d2[7];
 #pragma unroll
         for (int j = 0; j < 7; ++j) d2[j] = dist2_xy(P, idx[j], qh, ql, dz[j], status);
@@ -197,10 +188,9 @@ __device__ __forceinline__ int points_within(const PointSetK &P, float3 qh, floa
             constexpr int kSlot[7] = {5, 9, 6, 10, 1, 8, 4};
 #pragma unroll
             for (int j = 0; j < 7; ++j) pre[kSlot[j]] = d2[j];
-            const float zpp = __fadd_rn(zp, z0);
             const int32_t ix[5] = {im - c.G1, ip - c.G1, ip + c.G0 - c.G1, ip + c.G0, ip + 2 * c.G1};
-            const float dzx[5] = {__fsub_rn(zm, z1), __fsub_rn(zp, z1), __fsub_rn(zpp, z1), zpp,
-                                  __fadd_rn(__fadd_rn(zp, z1), z1)};
+            const float dzx[5] = {z_at(P, zb, -g0 - g1), z_at(P, zb, g0 - g1), z_at(P, zb, 2.0f * g0 - g1),
+                                  z_at(P, zb, 2.0f * g0), z_at(P, zb, g0 + 2.0f * g1)};
             constexpr int kSlotX[5] = {0, 2, 3, 7, 11};      // slot 14 is window candidate 11
 #pragma unroll
             for (int j = 0; j < 5; ++j) pre[kSlotX[j]] = dist2_xy(P, ix[j], qh, ql, dzx[j], status);
