@@ -21,6 +21,7 @@
 #include <math.h>
 
 #include "lf_device.cuh"
+#include "lf_df.cuh"
 #include "lf_kernels.h"
 
 namespace lfk {
@@ -240,36 +241,6 @@ __global__ void __launch_bounds__(256, kPreBlocks)
 // store 0. What bounds it, and the precompute: the FP32 pipe (73% of its cycles
 // with packed pairs at two cycles each, XU 58%, issue 73%).
 constexpr uint32_t kVolTileLog = 4;
-
-// Far end of the segment inside S from the front hit h along unit d: with f = h -
-// O, b = f . d and c = |f|^2 - R^2, -b + sqrt(b^2 - c). In FP32, c cancels for a
-// hit on S and b for a grazing ray; here f . d is summed in double-float and c is
-// error-free (the expansion of unit_hit_df), each then rounded once, so the
-// length is as exact as FP32 holds it. The same in FP64 (some forty operations and
-// a square root at a seventieth of FP32's rate), one launch per view and rows of
-// 256 pixels took 241 us for 8 views of 512^2, 62% hit; this takes 134.
-__device__ __forceinline__ float chord_length(const SphereK &S, float3 h, float3 d)
-{
-    const float hv[3] = {h.x, h.y, h.z}, dv[3] = {d.x, d.y, d.z};
-    df f[3], b{0.0f, 0.0f};
-    float small = 0.0f;
-    df sq{0.0f, 0.0f};
-#pragma unroll
-    for (int k = 0; k < 3; ++k) {
-        const df s = two_sum(hv[k], -S.o_hi[k]);
-        f[k] = fast_two_sum(s.h, __fsub_rn(s.l, S.o_lo[k]));
-        b = df_add(b, df_mul(f[k], df{dv[k], 0.0f}));
-        const float p = __fmul_rn(f[k].h, f[k].h);
-        small = __fadd_rn(small, __fmaf_rn(2.0f * f[k].h, f[k].l, __fmaf_rn(f[k].h, f[k].h, -p)));
-        const df t = two_sum(sq.h, p);
-        sq.h = t.h;
-        sq.l = __fadd_rn(sq.l, t.l);
-    }
-    const df r = two_sum(sq.h, -S.r2_h);
-    const float c = __fadd_rn(__fadd_rn(r.h, __fadd_rn(r.l, sq.l)), __fsub_rn(small, S.r2_l));
-    const float disc = __fmaf_rn(b.h, b.h, __fmaf_rn(2.0f * b.h, b.l, -c));
-    return disc > 0.0f ? fmaxf(0.0f, __fsub_rn(__fsqrt_rn(disc), b.h)) : 0.0f;
-}
 
 template <int MAXV>
 struct VolumeParams : PrecomputeParams {

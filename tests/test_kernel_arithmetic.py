@@ -22,6 +22,7 @@ static inline float __fsub_rn(float a, float b) { return a - b; }
 static inline float __fmul_rn(float a, float b) { return a * b; }
 static inline float __fmaf_rn(float a, float b, float c) { return std::fmaf(a, b, c); }
 static inline float __fsqrt_rn(float a) { return std::sqrt(a); }
+static inline float __frcp_rn(float a) { return 1.0f / a; }
 static inline float __int2float_rn(int a) { return (float)a; }
 #include "lf_df.cuh"
 
@@ -35,6 +36,21 @@ extern "C" void z_differences(uint32_t n, int64_t count, const float *qh, const 
         const lfk::ZOffset o = lfk::z_offset(P, b[q], qh[q], ql[q]);
         for (int j = 0; j < corners; ++j) out[q * corners + j] = lfk::z_at(P, o, (float)k[q * corners + j]);
     }
+}
+
+extern "C" void chord_lengths(double R, const double O[3], int64_t count, const float *h, const float *d, float *out)
+{
+    lfk::SphereK S{};
+    const double r2 = R * R;
+    S.r2_h = (float)r2;
+    S.r2_l = (float)(r2 - (double)S.r2_h);
+    for (int k = 0; k < 3; ++k) {
+        S.o_hi[k] = (float)O[k];
+        S.o_lo[k] = (float)(O[k] - (double)S.o_hi[k]);
+    }
+    for (int64_t i = 0; i < count; ++i)
+        out[i] = lfk::chord_length(S, make_float3(h[3 * i], h[3 * i + 1], h[3 * i + 2]),
+                                   make_float3(d[3 * i], d[3 * i + 1], d[3 * i + 2]));
 }
 """
 
@@ -97,3 +113,45 @@ def test_z_differences_of_the_corners(host, n):
     cached = ((qh[:, None] - ph) + (ql[:, None] - pl)).astype(np.float64)
     rms = np.sqrt(np.mean((err ** 2)[near])), np.sqrt(np.mean(((cached - want) ** 2)[near]))
     assert rms[0] <= 1.02 * rms[1], rms
+
+
+@pytest.mark.parametrize("R,O", [(1.0, (0.0, 0.0, 0.0)), (2.5, (0.4, -1.2, 0.7)), (0.37, (10.3, 20.1, -7.7)),
+                                 (1e-3, (0.0, 1e-3, 0.0)), (150.1, (1.0, 2.0, 3.0))])
+def test_chord_lengths(host, R, O):
+    """Central to grazing rays, from eyes 1.01 to 40 radii away: one rounding of the
+    length, and what 2^-43 of the squares it is formed from makes of it (each
+    double-float step is within 2^-46)."""
+    rng = np.random.default_rng(int(R * 1000))
+    n = 400_000
+    O = np.array(O)
+    e = random_queries(rng, n) * (R * np.exp(rng.uniform(np.log(1.01), np.log(40.0), n)))[:, None] + O
+    # aim at a point of the disc of S seen from the eye, half of them near its rim
+    axis = O - e
+    u = np.cross(axis, random_queries(rng, n))
+    u /= np.linalg.norm(u, axis=1, keepdims=True)
+    rim = np.where(rng.uniform(size=n) < 0.5, rng.uniform(0, 1, n), 1.0 - 10.0 ** rng.uniform(-5, -1, n))
+    L2 = (axis ** 2).sum(1)
+    d = axis + u * (rim * R / np.sqrt(L2 - R * R) * np.sqrt(L2))[:, None]
+    e32, d32 = e.astype(np.float32), (d / np.linalg.norm(d, axis=1, keepdims=True)).astype(np.float32)
+    # the front hit, rounded to FP32 as the camera step leaves it
+    f = e32.astype(np.float64) - O
+    b, c = (f * d32).sum(1), (f * f).sum(1) - R * R
+    hits = b * b > c * (d32.astype(np.float64) ** 2).sum(1)
+    tn = (-b - np.sqrt(np.maximum(b * b - c, 0.0))).astype(np.float32)
+    h = (e32 + (tn[:, None] * d32).astype(np.float32))[hits]
+    d32 = np.ascontiguousarray(d32[hits])
+    got = np.empty(len(h), np.float32)
+    host.chord_lengths(C.c_double(R), ptr(np.ascontiguousarray(O, np.float64)), C.c_int64(len(h)), ptr(h), ptr(d32), ptr(got))
+    w = np.longdouble
+    f = h.astype(w) - O.astype(w)
+    b, c = (f * d32.astype(w)).sum(1), (f * f).sum(1) - w(R) * w(R)
+    disc = b * b - c
+    inside = disc > 2.0 ** -30 * R * R          # a root whose argument is rounding only says nothing
+    assert inside.sum() > 300_000
+    root = np.sqrt(disc[inside])
+    want = np.maximum(root - b[inside], 0.0)
+    size = R * (R + np.abs(O).sum())
+    bound = 2.0 ** -24 * (1.0 + 2.0 ** -8) * want + 2.0 ** -43 * (size / root + size / R)
+    err = np.abs(got[inside] - want)
+    assert (err <= bound).all(), float((err / bound).max())
+    assert float(np.median(want)) > 0.1 * R
