@@ -358,7 +358,7 @@ template <int MAXV>
 static cudaError_t launch(const RenderParams<MAXV> &p, dim3 grid, unsigned block, cudaStream_t st)
 {
     void *args[] = {const_cast<RenderParams<MAXV> *>(&p)};
-    cudaError_t e = cudaLaunchKernel(backward_fn<MAXV>(p), grid, dim3(block), args, 0, st);
+    cudaError_t e = launch_kernel(backward_fn<MAXV>(p), grid, block, args, st);
     // nearest sampling may leave near-ties to the exact pass, an upper-hemisphere table rays at the rim of its rows
     if (e == cudaSuccess && !p.nine && !p.idx_in && (p.nearest_only || p.rows_stored)) e = launch_fixup(kF32C4, true, p, st);
     return e;

@@ -197,12 +197,14 @@ static cudaError_t launch(int kind, bool bwd, const RenderParams<MAXV> &p, cudaS
                 cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, f, (int)kFixupThreads, 0) == cudaSuccess &&
                 sms > 0 && per_sm > 0)
                 grids[slot] = (unsigned)(sms * per_sm);
+            else
+                cudaGetLastError();                      // the default grid serves
             dev_cached[slot] = dev;
         }
         grid = grids[slot];
     }
     void *args[] = {const_cast<RenderParams<MAXV> *>(&p)};
-    return cudaLaunchKernel(f, dim3(grid), dim3(kFixupThreads), args, 0, st);
+    return launch_kernel(f, dim3(grid), kFixupThreads, args, st);
 }
 
 cudaError_t launch_fixup(int kind, bool bwd, const RenderParams<kSmallViews> &p, cudaStream_t st)

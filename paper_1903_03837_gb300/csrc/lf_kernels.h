@@ -77,6 +77,15 @@ inline dim3 tile_grid(RenderParams<MAXV> &p)
     return p.grid3 ? dim3(tx, ty, p.n_views) : dim3(p.total_tiles);
 }
 
+// Launches kernel f; the error of a launch that fails goes to the caller and does
+// not stay behind for a later one to report.
+inline cudaError_t launch_kernel(const void *f, dim3 grid, unsigned block, void **args, cudaStream_t st)
+{
+    const cudaError_t e = cudaLaunchKernel(f, grid, dim3(block), args, 0, st);
+    if (e != cudaSuccess) cudaGetLastError();
+    return e;
+}
+
 // lf_render.cu: the forward launch (and, where it may queue rays, the exact pass).
 cudaError_t launch_render(int kind, const RenderParams<kSmallViews> &p, dim3 grid, unsigned block, cudaStream_t st);
 cudaError_t launch_render(int kind, const RenderParams<kLargeViews> &p, dim3 grid, unsigned block, cudaStream_t st);

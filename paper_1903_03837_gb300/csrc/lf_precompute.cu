@@ -296,7 +296,7 @@ static cudaError_t launch_volume(const VolumeParams<MAXV> &p, unsigned grid, cud
         (const void *)volume_direct_kernel<7, MAXV>, (const void *)volume_direct_kernel<8, MAXV>};
     static_assert(kMaxBlobs == 16, "pairs");
     void *args[] = {const_cast<VolumeParams<MAXV> *>(&p)};
-    return cudaLaunchKernel(f[p.nb ? (p.nb - 1) / 2 : 0], dim3(grid), dim3(256), args, 0, st);
+    return launch_kernel(f[p.nb ? (p.nb - 1) / 2 : 0], dim3(grid), 256, args, st);
 }
 
 template <int MAXV>
@@ -343,7 +343,7 @@ cudaError_t launch_precompute(const PrecomputeParams &p, cudaStream_t st)
     const uint64_t blocks = (total + 255) / 256;
     const unsigned grid = (unsigned)(blocks < (1ull << 20) ? blocks : (1ull << 20));
     void *args[] = {const_cast<PrecomputeParams *>(&p)};
-    return cudaLaunchKernel(f[p.nb ? (p.nb - 1) / 2 : 0], dim3(grid), dim3(256), args, 0, st);
+    return launch_kernel(f[p.nb ? (p.nb - 1) / 2 : 0], dim3(grid), 256, args, st);
 }
 
 }  // namespace lfk

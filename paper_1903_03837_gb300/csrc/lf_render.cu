@@ -225,7 +225,7 @@ template <int MAXV>
 static cudaError_t launch(int kind, const RenderParams<MAXV> &p, dim3 grid, unsigned block, cudaStream_t st)
 {
     void *args[] = {const_cast<RenderParams<MAXV> *>(&p)};
-    cudaError_t e = cudaLaunchKernel(render_fn<MAXV>(kind, p), grid, dim3(block), args, 0, st);
+    cudaError_t e = launch_kernel(render_fn<MAXV>(kind, p), grid, block, args, st);
     if (e == cudaSuccess && may_defer(p)) e = launch_fixup(kind, false, p, st);
     return e;
 }
