@@ -55,6 +55,7 @@
 
 #include "lf_device.cuh"
 #include "lf_kernels.h"
+#include "lf_post_plan.h"
 
 namespace lfk {
 
@@ -533,10 +534,10 @@ static void post_weight_image(const float *w, uint4 *img)
                 }
 }
 
-// Strips of 124 columns, chunks of chunk_rows rows (a multiple of kBand): the
-// chunks are as short as keeps the CTAs within one to four waves of the resident
-// slots (two per SM), at most 32 views of at most 65536 x 65536 pixels (fewer than
-// 2^31 CTAs). One wave leaves 18% of the slots empty on two 3840 x 2160 views.
+// Strips of 124 columns, chunks of chunk_rows rows (a multiple of kBand) by
+// post_chunk_bands over the resident slots (two per SM); at most 32 views of at most
+// 65536 x 65536 pixels (fewer than 2^31 CTAs). One wave leaves 18% of the slots empty
+// on two 3840 x 2160 views.
 cudaError_t launch_post_filter(const PostParams &p0, cudaStream_t st)
 {
     static thread_local PostK p;
@@ -593,39 +594,15 @@ cudaError_t launch_post_filter(const PostParams &p0, cudaStream_t st)
         memcpy(last_w, p0.w, sizeof last_w);
         have_image = true;
     }
-    uint64_t bands = 0, max_vb = 0, ctas = 0;
+    PostExtent extent[kPostMaxViews];
     for (uint32_t v = 0; v < p.n_views; ++v) {
         p.views[v] = p0.views[v];
         p.views[v].tiles_x = (p.views[v].width + kPW - 1) / kPW;
-        const uint64_t vb = (p.views[v].height + kBand - 1) / kBand;
-        bands += (uint64_t)p.views[v].tiles_x * vb;
-        max_vb = vb > max_vb ? vb : max_vb;
+        extent[v] = {p.views[v].tiles_x, (p.views[v].height + kBand - 1) / kBand};
     }
-    if (bands == 0) return cudaSuccess;
-    // the chunk length that fills one wave of the slots, two, three or four, whichever
-    // takes the fewest steps: a wave costs its chunk's bands, one more for the six rows
-    // before it and about as much again to start its CTAs
-    uint64_t per_chunk = max_vb;
-    double best = 1e300;
-    for (int waves = 1; waves <= 4; ++waves) {
-        const uint64_t slots = (uint64_t)cached_slots * waves;
-        uint64_t n = (bands + slots - 1) / slots;
-        for (; n < max_vb; ++n) {
-            ctas = 0;
-            for (uint32_t v = 0; v < p.n_views; ++v)
-                ctas += (uint64_t)p.views[v].tiles_x * ((p.views[v].height + kBand * n - 1) / (kBand * n));
-            if (ctas <= slots) break;
-        }
-        n = n < max_vb ? n : max_vb;
-        const double steps = waves * ((double)n + 2.3);
-        if (steps < best) {
-            best = steps;
-            per_chunk = n;
-        }
-        if (n == 1) break;
-    }
-    p.chunk_rows = (uint32_t)(per_chunk * kBand);
-    ctas = 0;
+    if (p.n_views == 0) return cudaSuccess;
+    p.chunk_rows = (uint32_t)(post_chunk_bands(extent, p.n_views, (uint64_t)cached_slots) * kBand);
+    uint64_t ctas = 0;
     for (uint32_t v = 0; v < p.n_views; ++v) {
         p.views[v].tiles_y = (p.views[v].height + p.chunk_rows - 1) / p.chunk_rows;
         p.tile_prefix[v] = (uint32_t)ctas;
