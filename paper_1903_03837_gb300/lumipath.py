@@ -169,23 +169,29 @@ def lf_create_table(desc: lf_table_desc, radiance_ptr: int, scales_ptr: Optional
     return int(h.value)
 
 
+# Device addresses go through c_void_p, which takes integers (and None) only: as a
+# bare argument ctypes would also pass the host address of bytes, a string or an array.
 def lf_render(table: int, views, n_views: int, out_ptr: int, idx_ptr: Optional[int], stream: int = 0):
-    _check((_lib or lib()).lf_render(table, views, n_views, out_ptr, idx_ptr or None, stream or None))
+    _check(lib().lf_render(C.c_void_p(table), views, n_views, C.c_void_p(out_ptr),
+                           C.c_void_p(idx_ptr or None), C.c_void_p(stream or None)))
 
 
 def lf_render_f16(table: int, views, n_views: int, out_ptr: int, idx_ptr: Optional[int], stream: int = 0):
-    _check((_lib or lib()).lf_render_f16(table, views, n_views, out_ptr, idx_ptr or None, stream or None))
+    _check(lib().lf_render_f16(C.c_void_p(table), views, n_views, C.c_void_p(out_ptr),
+                               C.c_void_p(idx_ptr or None), C.c_void_p(stream or None)))
 
 
 def lf_render_backward(table: int, views, n_views: int, grad_out_ptr: int, grad_table_ptr: int,
                        stream: int = 0):
-    _check((_lib or lib()).lf_render_backward(table, views, n_views, grad_out_ptr, grad_table_ptr, stream or None))
+    _check(lib().lf_render_backward(C.c_void_p(table), views, n_views, C.c_void_p(grad_out_ptr),
+                                    C.c_void_p(grad_table_ptr), C.c_void_p(stream or None)))
 
 
 def lf_render_backward_idx(table: int, views, n_views: int, grad_out_ptr: int, idx_ptr: int,
                            grad_table_ptr: int, stream: int = 0):
-    _check((_lib or lib()).lf_render_backward_idx(table, views, n_views, grad_out_ptr, idx_ptr, grad_table_ptr,
-                                                  stream or None))
+    _check(lib().lf_render_backward_idx(C.c_void_p(table), views, n_views, C.c_void_p(grad_out_ptr),
+                                        C.c_void_p(idx_ptr), C.c_void_p(grad_table_ptr),
+                                        C.c_void_p(stream or None)))
 
 
 def lf_destroy(table: Optional[int]):
@@ -213,7 +219,8 @@ def lf_sync_status(table: int, stream: int = 0):
 
 def lf_quantize_table(src_ptr: int, M: int, N: int, Cc: int, dtype: int, codes_ptr: int,
                       scales_ptr: int, stream: int = 0):
-    _check((_lib or lib()).lf_quantize_table(src_ptr, M, N, Cc, dtype, codes_ptr, scales_ptr, stream or None))
+    _check(lib().lf_quantize_table(C.c_void_p(src_ptr), M, N, Cc, dtype, C.c_void_p(codes_ptr),
+                                   C.c_void_p(scales_ptr), C.c_void_p(stream or None)))
 
 
 def lf_fill_lobe_table(M: int, N: int, Cc: int, L: int, ap, ad, kp, kd, col, noise_seed: int,
@@ -244,13 +251,14 @@ def lf_noalloc_sync_status(stream: int = 0):
 
 def lf_precompute_table(desc: lf_precompute_desc, blobs, out_ptr: int, stream: int = 0):
     """Light-field precompute of a volume scene into a device FP32 table (Section 2)."""
-    _check((_lib or lib()).lf_precompute_table(C.byref(desc), blobs, out_ptr, stream or None))
+    _check(lib().lf_precompute_table(C.byref(desc), blobs, C.c_void_p(out_ptr), C.c_void_p(stream or None)))
 
 
 def lf_render_volume(desc: lf_precompute_desc, blobs, views, n_views: int, out_ptr: int, stream: int = 0):
     """Direct render of the precompute's volume along each pixel's ray (the
     ground truth of a light-field render of the precomputed table)."""
-    _check((_lib or lib()).lf_render_volume(C.byref(desc), blobs, views, n_views, out_ptr, stream or None))
+    _check(lib().lf_render_volume(C.byref(desc), blobs, views, n_views, C.c_void_p(out_ptr),
+                                  C.c_void_p(stream or None)))
 
 
 LF_POST_WEIGHTS = 3347
@@ -261,8 +269,8 @@ def lf_post_filter(radius: float, center, channels: int, weights_host, views, n_
     """Learned post-filter of a light-field image (three 3x3 convolution layers,
     residual on hit pixels); weights_host: a ctypes array of LF_POST_WEIGHTS floats."""
     c = (C.c_double * 3)(*[float(x) for x in center])
-    _check((_lib or lib()).lf_post_filter(float(radius), c, channels, weights_host, views, n_views, in_ptr, out_ptr,
-                                          stream or None))
+    _check(lib().lf_post_filter(float(radius), c, channels, weights_host, views, n_views, C.c_void_p(in_ptr),
+                                C.c_void_p(out_ptr), C.c_void_p(stream or None)))
 
 
 def lf_device_sm_count() -> int:
