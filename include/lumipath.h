@@ -274,11 +274,12 @@ lf_status lf_precompute_table(const lf_precompute_desc *desc, const lf_blob *blo
  * ray is then integrated as above from h_o along its direction to the far
  * intersection with S (that length by double-float sums), one sample, no jitter.
  * out_dev [pixels][channels] FP32 (device, caller-owned; RGB, plus opacity
- * 1 - T for channels = 4), written at each view's out_offset; misses store 0.
+ * 1 - T for channels = 4), written at each view's out_offset (of views that
+ * overlap there the last one stays); misses store 0.
  * Reads radius, center, channels, steps, n_blobs and the background of
  * `desc`; n_origins, n_directions, rows, spp, jitter and seed are ignored.
  * out_dev must be 16-byte aligned for 4 channels, 4-byte for 3. One kernel
- * launch per 32 views; allocates nothing. Errors: LF_ERR_INVALID_ARG (NULL,
+ * launch per 32 views that do not overlap; allocates nothing. Errors: LF_ERR_INVALID_ARG (NULL,
  * ranges, non-finite values, views as for lf_render), LF_ERR_CUDA.
  * Asynchronous on `stream`. */
 lf_status lf_render_volume(const lf_precompute_desc *desc, const lf_blob *blobs_host,

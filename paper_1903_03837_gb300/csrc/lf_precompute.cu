@@ -299,6 +299,12 @@ static cudaError_t launch_volume(const VolumeParams<MAXV> &p, unsigned grid, cud
     return launch_kernel(f[p.nb ? (p.nb - 1) / 2 : 0], dim3(grid), 256, args, st);
 }
 
+static bool output_overlap(const ViewK &a, const ViewK &b)
+{
+    const uint64_t ea = a.out_offset + (uint64_t)a.width * a.height, eb = b.out_offset + (uint64_t)b.width * b.height;
+    return a.out_offset < eb && b.out_offset < ea;
+}
+
 template <int MAXV>
 static cudaError_t launch_views(const PrecomputeParams &base, const SphereK &S, const lf_view *views, uint32_t n,
                                 double R, const double O[3], cudaStream_t st)
@@ -308,13 +314,18 @@ static cudaError_t launch_views(const PrecomputeParams &base, const SphereK &S, 
     p.sphere = S;
     lf_launch tile = {1u << kVolTileLog, 1u << kVolTileLog, 8, 0, 0, 0};
     for (uint32_t v0 = 0; v0 < n;) {
-        // as many views as the parameters hold and a grid of fewer than 2^31 tiles
+        // as many views as the parameters hold, a grid of fewer than 2^31 tiles, and no
+        // view that overlaps an earlier one of the launch in the output: the last one
+        // stays there, as if each view had its own launch
         uint64_t tiles = 0;
         uint32_t nv = 0;
         for (; nv < (uint32_t)MAXV && v0 + nv < n; ++nv) {
             p.views[nv] = view_params(views[v0 + nv], tile, R, O);
             const uint64_t t = (uint64_t)p.views[nv].tiles_x * p.views[nv].tiles_y;
             if (nv && tiles + t >= (1ull << 31)) break;
+            bool overlaps = false;
+            for (uint32_t k = 0; k < nv; ++k) overlaps |= output_overlap(p.views[k], p.views[nv]);
+            if (overlaps) break;
             p.tile_prefix[nv] = (uint32_t)tiles;
             tiles += t;
         }
