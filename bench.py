@@ -811,8 +811,7 @@ def run_batching(args):
     codes, s = api.quantize_table(T32, "f16")
     del T32
     lf = api.LightField(codes, "f16", s, borrow=True)
-    persistent = [c for c in autotune.CANDIDATES if c[4] == 1]
-    ranked = autotune.tune(lf, [cfg.views], persistent, reps=2)
+    ranked = autotune.tune(lf, [cfg.views], reps=2)
     launch = ranked[0][1]
     lf.set_launch(**launch)
     out = torch.empty((cfg.rays, 4), device="cuda")

@@ -1,8 +1,7 @@
 """Launch-shape autotuner for the render kernel.
 
-Times candidate launch shapes (CTA tile, warp sub-tile, tile order, static or
-persistent grid) on the caller's own views with CUDA events and keeps the
-fastest. Results are cached per (key, device name) in a JSON file next to the
+Times candidate launch shapes (CTA tile, warp sub-tile, tile order) on the
+caller's own views with CUDA events and keeps the fastest. Results are cached per (key, device name) in a JSON file next to the
 built library, so a workload is tuned once per machine.
 """
 from __future__ import annotations
@@ -17,14 +16,14 @@ from . import build as _build
 CACHE = os.path.join(_build.BUILD, "autotune.json")
 _lock = threading.Lock()
 
-# (tile_w, tile_h, warp_w, order, persistent; the last has no effect on a launch)
+# (tile_w, tile_h, warp_w, order, persistent); persistent has no effect on a launch, so
+# it is 0 throughout and no two candidates are the same launch
 CANDIDATES = [
-    (16, 16, 8, 0, 0), (16, 16, 8, 1, 0), (16, 16, 8, 0, 1), (16, 16, 8, 1, 1),
-    (32, 8, 8, 0, 0), (32, 8, 8, 1, 1), (8, 32, 8, 0, 0), (16, 8, 8, 0, 0),
-    (16, 16, 16, 0, 0), (32, 8, 32, 0, 0), (16, 16, 4, 0, 0), (64, 4, 8, 1, 1),
-    (32, 4, 8, 0, 0), (8, 16, 8, 1, 1), (16, 8, 4, 0, 0),
+    (16, 16, 8, 0, 0), (16, 16, 8, 1, 0), (32, 8, 8, 0, 0), (32, 8, 8, 1, 0), (8, 32, 8, 0, 0), (16, 8, 8, 0, 0),
+    (16, 16, 16, 0, 0), (32, 8, 32, 0, 0), (16, 16, 4, 0, 0), (64, 4, 8, 1, 0), (32, 4, 8, 0, 0), (8, 16, 8, 1, 0),
+    (16, 8, 4, 0, 0),
 ]
-QUICK = [(16, 16, 8, 0, 0), (16, 16, 8, 1, 1), (32, 8, 8, 0, 0), (16, 8, 8, 0, 0)]
+QUICK = [(16, 16, 8, 0, 0), (16, 16, 8, 1, 0), (32, 8, 8, 0, 0), (16, 8, 8, 0, 0)]
 
 
 def as_launch(c) -> Dict[str, int]:
