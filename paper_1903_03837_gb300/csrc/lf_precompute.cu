@@ -54,7 +54,8 @@ __device__ __forceinline__ float2 add2(float2 a, float2 b)
 }
 
 // (1 - exp(-x)) / x = 1 + x P(x) on [0, 1], P of degree 5 by interpolation at the
-// Chebyshev nodes (within 4e-8 of it in exact arithmetic, 1e-7 in float32). With
+// Chebyshev nodes (fit_step_weight.py writes the coefficients: within 4e-8 of it in
+// exact arithmetic, 1e-7 in float32). With
 // T e^-x = T - w x it replaces the exponential of a step's optical depth: two ex2
 // and a division less per step, and without their error, which the transmittance
 // multiplied up, the table is within 1e-7 (relative norm) of 64 bits instead of
