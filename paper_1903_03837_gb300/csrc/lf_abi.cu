@@ -512,7 +512,6 @@ lf_status lf_create_table(const lf_table_desc *d, const void *radiance_dev, cons
     t->rows = rows;
     t->launch = default_launch();
     cudaGetDevice(&t->device);
-    t->sm_count = lf_device_sm_count();
     cudaStream_t st = (cudaStream_t)stream;
     cudaError_t e;
     auto bail = [&](lf_status s) { lf_destroy(t); return s; };

@@ -44,7 +44,7 @@ struct ViewK {
     uint32_t outside;
     float q[6];              // certain_miss: q0 + q1 x + q2 y + q3 x^2 + q4 x y + q5 y^2 < 0 at pixel (x, y)
     // Pixels outside columns [sx0, sx1) or rows [sy0, sy1) certainly miss S
-    // (the screen bound of certain_miss, widened by two pixels).
+    // (the screen bound of certain_miss, widened by three pixels).
     uint32_t sx0, sx1, sy0, sy1;
     // lt / tiles_x for any lt < 2^31 is (lt * div_m) >> div_s (64-bit product)
     uint32_t div_m, div_s;
@@ -128,5 +128,4 @@ struct lf_table {
     lfk::SphereK sphere;
     lfk::PointSetK po, pd;
     lf_launch launch;
-    int sm_count;
 };
