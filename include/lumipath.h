@@ -162,9 +162,12 @@ lf_status lf_render_backward(const lf_table *t, const lf_view *views_host, uint3
 /* The same gradient from the sample indices a render of the same views wrote
  * (idx_dev: device int32 [P][2K] as lf_render writes them, [P][2] with nearest
  * sampling), instead of a new index step: the hits, the unit hits and the
- * double-float distances of these indices are recomputed, the same distances by
- * the same function as the index step's, so the weights are identical and a
- * fit that keeps its forward indices skips the search in the backward. A miss
+ * distances of these indices are recomputed. The weights agree with the render's
+ * within 5e-6 (each side rounds the distances in FP32 in its own way). Which route
+ * is cheaper: with 5 or 9 neighbours an image without indices and
+ * lf_render_backward, whose searches need no ranking (118 us together for a 1080p
+ * view of a 65,536 x 1,024 table, against 190 for a render with indices and this
+ * call); with nearest sampling, or where the indices are kept anyway, this one. A miss
  * (index -1) contributes nothing; an index out of range counts as missing and
  * makes the next lf_sync_status report LF_ERR_DEVICE_CHECK.
  * Errors: LF_ERR_INVALID_ARG, LF_ERR_CUDA. */

@@ -10,9 +10,9 @@
 //   G[a][b] = sum over rays r of wo[a][r] wd[b][r] g[r]
 // divided over the lanes, a pair (a, b) at a time: one atomic per texel and warp.
 // On the fit of 32 views of 512^2 into a 16,384 x 512 table I is 5 to 8 and J 3
-// to 5: 0.36 ms for its 8.4 M rays (68% hit), search included, where 25 taps a ray
+// to 5: 0.35 ms for its 8.4 M rays (68% hit), search included, where 25 taps a ray
 // of ballots, shuffles and group sums took 0.93 from the forward's indices and
-// more with a search. Issue-bound (73% of the slots, ALU pipe 49%, FMA 36%).
+// more with a search. Issue-bound (73% of the slots, ALU pipe 56%, FMA 32%).
 // Warps with more distinct neighbours than kMaxO or kMaxD (small views of large
 // tables) sum tap by tap over the lanes that share a texel: a dense matrix would
 // hold mostly zeros.
@@ -21,7 +21,7 @@
 #include "lf_ray.cuh"
 
 // Resident CTAs of kMaxBlock threads per SM the register budget is cut for: the
-// fit's forward and backward take 631 us at 5, 640 at 4, 35 more at 3.
+// fit's forward and backward took 631 us at 5 (now 643), 640 at 4, 35 more at 3.
 #ifndef LF_MIN_BLOCKS_BWD
 #define LF_MIN_BLOCKS_BWD 5
 #endif

@@ -56,10 +56,11 @@ __device__ __forceinline__ float2 add2(float2 a, float2 b)
 // (1 - exp(-x)) / x = 1 + x P(x) on [0, 1], P of degree 5 by interpolation at the
 // Chebyshev nodes (fit_step_weight.py writes the coefficients: within 4e-8 of it in
 // exact arithmetic, 1e-7 in float32). With
-// T e^-x = T - w x it replaces the exponential of a step's optical depth: two ex2
-// and a division less per step, and without their error, which the transmittance
-// multiplied up, the table is within 1e-7 (relative norm) of 64 bits instead of
-// 6 to 8e-7.
+// T e^-x = T - w x it takes the place of the exponential of a step's optical depth:
+// without that one's error, which the transmittance multiplied up, the table is
+// within 1.3e-7 (relative norm) of 64 bits instead of 6 to 8e-7. It spares no XU
+// instruction: the dense step's ex2 and reciprocal (past x = 1) are issued in every
+// step, 10.1 of them a step for 8 blobs, 50.7 instructions in all (51.7 before).
 __device__ __forceinline__ float one_minus_exp_over_x(float x)
 {
     float h = 0.00013742418377660215f;
@@ -74,8 +75,8 @@ __device__ __forceinline__ float one_minus_exp_over_x(float x)
 // CTAs of 256 threads per SM the register budget is cut for (the direct render of 9
 // blobs or more: 2), and the unroll of the step loop. Precompute of 16,384 x 512 texels,
 // 8 blobs, 4 samples of 64 steps: 3.73 ms at 2 and 2, 3.75 to 3.82 at 3 or 4 CTAs
-// or unrolled by 1 or 4. Direct render of 8 views of 512^2: 134 us at 3 and 4, 136
-// to 140 elsewhere. Scalar instead of packed FP32 costs the precompute 10% and
+// or unrolled by 1 or 4. Direct render of 8 views of 512^2: 133 us at 3 and 4, 1
+// to 4% more elsewhere. Scalar instead of packed FP32 costs the precompute 10% and
 // more.
 constexpr int kPreBlocks = 2, kPreUnroll = 2, kVolBlocks = 3, kVolUnroll = 4;
 
@@ -239,8 +240,10 @@ __global__ void __launch_bounds__(256, kPreBlocks)
 // camera ray and its front hit h_o on S (the FP32 steps of the light-field
 // render), the length of the ray inside S from h_o (chord_length), then the
 // integral of the precompute along that ray (one sample, no jitter). Misses
-// store 0. What bounds it, and the precompute: the FP32 pipe (73% of its cycles
-// with packed pairs at two cycles each, XU 58%, issue 73%).
+// store 0. What bounds it, and the precompute: the FP32 pipe (70 and 73% of its
+// cycles, with packed pairs at two cycles each), XU (54 and 59%) and issue (73%)
+// together. 8 views of 512^2, 62% hit: 133 us; the chord in FP64, one launch a view
+// and rows of 256 pixels took 241.
 constexpr uint32_t kVolTileLog = 4;
 
 template <int MAXV>

@@ -12,24 +12,25 @@
 // instead, one barrier and one shared word per tile: 18% slower on 64 uneven
 // views (4.10 against 3.46 ms), so a launch is never persistent.
 //
-// What bounds it: instruction issue (75% of the issue slots on a 1080p frame of
-// a 65,536 x 1,024 FP16 table, ALU pipe 46%, FMA 38%, DRAM 3%). An image lists
+// What bounds it: instruction issue (79% of the issue slots on a 1080p frame of
+// a 65,536 x 1,024 FP16 table, ALU pipe 48%, FMA 39%, DRAM 3%). An image lists
 // the points within the kernel's radius (lf_ray.cuh) instead of ranking the
-// nearest ones and certifying the order: that frame 0.051 ms instead of 0.119
-// (1,430 thread instructions per hit ray instead of 2,680, and no exact pass), a
-// 2 x 3840 x 2160 frame of a 262,144 x 4,096 E4M3 table 0.252 instead of 0.547,
-// 64 uneven views of a 16,384 x 512 FP16 table 3.19 instead of 6.46. Per hit ray of
-// that frame: blend 381, candidates' distances 250, lattice corners 267, unit hits
-// 182, camera and hits 107, lists 76.
+// nearest ones and certifying the order: that frame 0.050 ms instead of 0.119
+// (1,420 thread instructions per hit ray instead of 2,680, and no exact pass), a
+// 2 x 3840 x 2160 frame of a 262,144 x 4,096 E4M3 table 0.258 instead of 0.547,
+// 64 uneven views of a 16,384 x 512 FP16 table 3.29 instead of 6.46. Per hit ray of
+// that frame, counted before the corners' z differences were rounded once: blend
+// 381, candidates' distances 250, lattice corners 267, unit hits 182, camera and
+// hits 107, lists 76.
 #include <cuda_fp16.h>
 #include <cuda_runtime.h>
 
 #include "lf_ray.cuh"
 
 // Resident CTAs of kMaxBlock threads per SM the register budget of the unranked
-// kernels is cut for: 5 (48 registers, 8 bytes spilled) against 4 takes the 4K
-// stereo frame from 277 to 252 us and the 64 views from 3.29 to 3.19 ms; 6 is 2%
-// slower than 5. The variants that rank 5 indices spill 80 bytes at 4.
+// kernels is cut for: 5 (48 registers, 12 to 24 bytes spilled) against 4 took the 4K
+// stereo frame from 277 to 252 us and the 64 views from 3.29 to 3.19 ms; 6 was 2%
+// slower than 5. The variants that rank 5 indices spill 130 bytes at 4.
 #ifndef LF_MIN_BLOCKS
 #define LF_MIN_BLOCKS 5
 #endif
